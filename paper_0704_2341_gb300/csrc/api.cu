@@ -2,7 +2,7 @@
 // wilson_apply, permute_sites, schur_apply and schur_solve.
 #include <math.h>
 
-#include "gs_internal.cuh"
+#include "fx.cuh"
 
 using namespace gs;
 
@@ -99,6 +99,8 @@ gs_status gs_create(gs_ctx** out, const int dims[4], double m0, void* stream) {
     }
     const size_t vbytes = (size_t)V * kSiteC * sizeof(double2);
     bool ok = cudaMalloc(&c->U_abi, (size_t)V * 36 * sizeof(double2)) == cudaSuccess &&
+              cudaMalloc(&c->fx_m, (size_t)fx_padded(V) * kSiteC * sizeof(longlong2)) == cudaSuccess &&
+              cudaMalloc(&c->fx_e, (size_t)V * sizeof(int)) == cudaSuccess &&
               cudaMalloc(&c->full_a, vbytes) == cudaSuccess &&
               cudaMalloc(&c->full_b, vbytes) == cudaSuccess &&
               cudaMalloc(&c->full_c, vbytes) == cudaSuccess &&
@@ -136,6 +138,7 @@ gs_status gs_destroy(gs_ctx* c) {
     free_net_ctx(c);
     free_mixed(c);
     free_persist(c);
+    free_persist_fx(c);
     for (cudaEvent_t e : c->prof.ev) cudaEventDestroy(e);
     c->prof.ev.clear();
     cudaFree(c->prof.ran_dev);
@@ -144,6 +147,8 @@ gs_status gs_destroy(gs_ctx* c) {
     for (Plan* p : c->plans) free_plan(p);
     c->plans.clear();
     cudaFree(c->U_abi);
+    cudaFree(c->fx_m);
+    cudaFree(c->fx_e);
     cudaFree(c->full_a);
     cudaFree(c->full_b);
     cudaFree(c->full_c);

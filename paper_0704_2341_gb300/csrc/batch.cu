@@ -13,10 +13,14 @@
 // a few solves side by side fill those gaps (24^3 x 48, FP32 inner: 5.87 s per
 // solve alone, 5.49 / 5.31 / 5.26 / 5.32 s with 2 / 3 / 4 / 6 at once, so four
 // lanes by default).  The cooperative grids of the running solves are drawn
-// from one block ledger (BlockLedger): every persistent solver kernel has the
-// same block footprint (128 threads, 168 registers), a grid is granted only
-// from blocks no other solve holds, so all of them stay co-resident, and the
-// blocks a finished solve frees go to the next launches of the others.
+// from one block ledger (BlockLedger): all cooperative blocks of a call have one
+// size (its inner precision and the sizes of its lattices pick one kernel), a
+// grid is granted only from blocks no other solve holds, so all of them stay
+// co-resident, and the blocks a finished solve frees go to the next launches of
+// the others.  On small lattices the FP64 solver's blocks keep their tile on
+// chip and are granted a whole grid at a time; a finished launch gives them back
+// at once (four permutations of 8^4: 126 ms against 154 with even shares of
+// blocks that keep their vectors in memory).
 #include <algorithm>
 #include <chrono>
 #include <condition_variable>
@@ -116,9 +120,8 @@ void ledger_leave(BlockLedger* L, const gs_ctx* c) {
     L->cv.notify_all();
 }
 
-int64_t ledger_grant(gs_ctx* c, int per_sm, int64_t want, int64_t target) {
+int64_t ledger_grant(gs_ctx* c, int64_t capacity, int64_t want, int64_t target, int64_t least) {
     BlockLedger* L = c->ledger;
-    const int64_t capacity = (int64_t)per_sm * c->num_sms;
     int64_t limit = want < target ? want : target;
     if (limit < 1) limit = 1;
     std::unique_lock<std::mutex> lk(L->mu);
@@ -138,8 +141,8 @@ int64_t ledger_grant(gs_ctx* c, int per_sm, int64_t want, int64_t target) {
                 claimed += e.launched ? e.blocks : (e.blocks > L->reserve ? e.blocks : L->reserve);
             }
         int64_t g = limit < capacity - claimed ? limit : capacity - claimed;
-        if (g < 1) g = limit < capacity - held ? limit : capacity - held;
-        if (g >= 1) {
+        if (g < least) g = limit < capacity - held ? limit : capacity - held;
+        if (g >= least) {
             mine->blocks = g;
             mine->launched = true;
             L->cv.notify_all();   // a solve waiting for blocks may find some now
@@ -152,6 +155,17 @@ int64_t ledger_grant(gs_ctx* c, int per_sm, int64_t want, int64_t target) {
         for (auto& e : L->held)
             if (e.ctx == c) mine = &e;
     }
+}
+
+void ledger_release(gs_ctx* c) {
+    BlockLedger* L = c->ledger;
+    if (!L) return;
+    {
+        std::lock_guard<std::mutex> lk(L->mu);
+        for (auto& e : L->held)
+            if (e.ctx == c) e.blocks = 0;
+    }
+    L->cv.notify_all();
 }
 
 }  // namespace gs
@@ -203,6 +217,13 @@ gs_status schur_solve_batched(int nprob, gs_ctx* const* ctxs, const int* type, c
     // a solve that has not launched yet is counted at a third of an even
     // share of the co-resident blocks (one block per SM share at 3 per SM)
     ledger.reserve = std::max(1, ctxs[0]->num_sms / std::max(1, lanes));
+    // the on-chip FP64 solver's grids are granted whole: the largest rest set
+    // (15/16 of a lattice, Type I) has to leave room for another solve
+    ledger.resident = true;
+    for (int i = 0; i < nprob; ++i) {
+        const int64_t rest = type[i] == GS_TYPE_I ? ctxs[i]->V - ctxs[i]->V / 16 : ctxs[i]->V / 2;
+        if (rest > 32ll * ctxs[i]->num_sms || ctxs[i]->opt_coop_blocks > 0) ledger.resident = false;
+    }
     size_t left = items.size();
 
     auto lane = [&]() {

@@ -1,5 +1,6 @@
-// Device code of the FP64 Wilson stencil, shared by the stand-alone stencil
-// kernel (dslash_f64.cu) and the persistent solver kernels (persistent.cu).
+// Device code of the Wilson stencil in double precision: the kernel of the entry
+// point that allocates nothing (dslash_f64.cu), the tiles that fixed point cannot
+// hold (dslash_fx.cuh) and the solver of such problems (persistent.cu).
 #pragma once
 
 #include "gs_internal.cuh"
@@ -139,7 +140,8 @@ __device__ __forceinline__ void hop_mu(const StencilArgs& a, int64_t j, bool val
 }
 
 
-// One tile of ts <= 32 output sites (lane l < ts handles site base + l):
+// One tile of ts <= 32 output sites (lane l < ts handles site base + l), by the
+// block's first four warps (all of them meet its barriers):
 // phase 1 (warp w = direction w, both hops, to shared memory) and phase 2
 // (warp w sums spin component w, adds the diagonal term, negation and addend,
 // stores, and accumulates the epilogue dots into e).
@@ -151,7 +153,7 @@ __device__ __forceinline__ void f64_tile(const StencilArgs& a, int64_t base, int
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
         // phase 1: warp `warp` computes direction mu = warp for the tile's sites
-    {
+    if (warp < 4) {
         const int64_t k = base + lane;
         const bool valid = lane < ts && k < a.n_out;
         const int64_t j = a.o0 + k;
@@ -174,7 +176,7 @@ __device__ __forceinline__ void f64_tile(const StencilArgs& a, int64_t base, int
     }
     __syncthreads();
     // phase 2: warp w finishes spin component w of the tile's sites
-    {
+    if (warp < 4) {
         const int spin = warp;
         const int64_t k = base + lane;
         if (lane < ts && k < a.n_out) {
@@ -223,6 +225,103 @@ __device__ __forceinline__ void f64_tile(const StencilArgs& a, int64_t base, int
         }
     }
     __syncthreads();
+}
+
+// Block sums of the epilogue dots, finished by the last block of the grid
+// (alpha = rho / <rhat, v> or omega = <t, s> / <t, t>).
+template <int EPI, int THREADS>
+__device__ __forceinline__ void stencil_finish(const StencilArgs& a, const double (&e)[5]) {
+    __shared__ double bred[THREADS / 32][kMaxRedVals];
+    const int warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    double e0 = e[0], e1 = e[1], e2 = e[2];
+
+    if constexpr (EPI == EPI_NONE) {
+        return;
+    } else {
+
+    auto warps = [&](int q) {
+        double s = 0.0;
+#pragma unroll
+        for (int w = 0; w < THREADS / 32; w += 4)
+            s += (bred[w][q] + bred[w + 1][q]) + (bred[w + 2][q] + bred[w + 3][q]);
+        return s;
+    };
+    // block reduction of the epilogue sums, then the last block finishes
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        e0 += __shfl_xor_sync(0xffffffffu, e0, off);
+        e1 += __shfl_xor_sync(0xffffffffu, e1, off);
+        e2 += __shfl_xor_sync(0xffffffffu, e2, off);
+    }
+    if (lane == 0) {
+        bred[warp][0] = e0;
+        bred[warp][1] = e1;
+        bred[warp][2] = e2;
+    }
+    __syncthreads();
+    __shared__ bool am_last;
+    if (threadIdx.x == 0) {
+        double* part = a.red.partial + (int64_t)blockIdx.x * kMaxRedVals;
+        part[0] = warps(0);
+        part[1] = warps(1);
+        part[2] = warps(2);
+        __threadfence();
+        const unsigned prev = atomicAdd(a.red.counter, 1u);
+        am_last = (prev == gridDim.x - 1);
+    }
+    __syncthreads();
+    if (!am_last) return;
+    __threadfence();
+    // deterministic: fixed per-thread strides then a fixed tree
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += THREADS) {
+        const volatile double* part = a.red.partial + (int64_t)b * kMaxRedVals;
+        s0 += part[0];
+        s1 += part[1];
+        s2 += part[2];
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, off);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, off);
+    }
+    if (lane == 0) {
+        bred[warp][0] = s0;
+        bred[warp][1] = s1;
+        bred[warp][2] = s2;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s0 = warps(0);
+        s1 = warps(1);
+        s2 = warps(2);
+        BicgState* st = a.st;
+        if (EPI == EPI_DOT_RHAT_V) {
+            const double2 den = make_double2(s0, s1);
+            if (den.x == 0.0 && den.y == 0.0) {
+                st->status = GS_BREAKDOWN;
+                st->done = 1;
+            } else {
+                st->alpha = cdiv(st->rho, den);
+                if (!isfinite(st->alpha.x) || !isfinite(st->alpha.y)) {
+                    st->status = GS_NONFINITE;
+                    st->done = 1;
+                }
+            }
+        } else {
+            // omega = <t,s>/<t,t>; t == 0 means s == 0 (D_rr is regular): omega = 0
+            st->omega = (s2 > 0.0) ? make_double2(s0 / s2, s1 / s2) : make_double2(0.0, 0.0);
+            if (!isfinite(st->omega.x) || !isfinite(st->omega.y)) {
+                st->status = GS_NONFINITE;
+                st->done = 1;
+            }
+        }
+        if (st->done) publish(st);
+        *a.red.counter = 0u;
+    }
+    }
 }
 
 }  // namespace

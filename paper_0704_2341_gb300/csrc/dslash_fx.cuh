@@ -1,0 +1,287 @@
+// Device code of the Wilson stencil in block fixed point (fx.cuh): a block of 16
+// warps computes a tile of up to 32 output sites.  The double-precision tile
+// (dslash_f64.cuh) takes over for a tile whose inputs fixed point cannot hold.
+#pragma once
+
+#include "dslash_f64.cuh"
+#include "fx.cuh"
+
+namespace gs {
+namespace {
+
+// NS = spin components of the two-spinor per thread: 1 (16 warps a tile, the
+// shortest tile) or 2 (8 warps, fewer instructions a site)
+template <int NS>
+constexpr int kFxThreads = 512 / NS;
+constexpr int kFxRow = 3;   // complex numbers in a site's row of a hop component (odd: free of bank conflicts)
+
+union FxShared {
+    longlong2 hop[16][kSitesPerBlock][kFxRow];   // [4 mu + 2 backward + two-spinor component][site][colour]
+    double f64[4][24][kSitesPerBlock];
+};
+
+struct I2 {  // re, im
+    long long x, y;
+};
+__device__ __forceinline__ I2 operator+(I2 a, I2 b) { return I2{a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ I2 operator-(I2 a, I2 b) { return I2{a.x - b.x, a.y - b.y}; }
+__device__ __forceinline__ I2 fx_add_i(I2 a, I2 b) { return I2{a.x - b.y, a.y + b.x}; }   // a + i b
+__device__ __forceinline__ I2 fx_sub_i(I2 a, I2 b) { return I2{a.x + b.y, a.y - b.x}; }   // a - i b
+
+// A thread's share of a hop: NS spin components of the projected two-spinor h =
+// psi_up -+ X_mu psi_lo of one input site, times the link, in units of
+// 2^(E - 1022 - 57); sh = E - the input site's exponent.  Stored is g = U h for a
+// forward hop and conj(g), g = U^dag h, for a backward one: with h conjugated as
+// well the backward product is U^T conj(h), so one piece of code serves all warps
+// and the SM shares its instruction lines (eight specialised copies starved on
+// instruction fetch).  Only the projection and the order of the link's entries
+// branch on the hop w = 4 mu + 2 backward + first component.
+template <int NS>
+struct FxOperands {
+    int4 u[9];                      // [c][r]: U for the forward hop, its transpose for the backward one
+    longlong2 s[NS][3], q[NS][3];   // upper spin components and their partners among the lower ones
+};
+
+// X_mu pairs spins 0, 1 with 3, 2 (mu < 2) or 2, 3
+__device__ __forceinline__ int fx_partner(int w, int s) { return ((w < 8) != (s != 0)) ? 9 : 6; }
+
+template <int NS, bool CG>
+__device__ __forceinline__ void fx_load_spinor(const StencilArgs& a, int w, int in, FxOperands<NS>& o) {
+    const longlong2* p = a.fxm + fx_index(in, kSiteC);
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+        const int s = (NS == 1 ? (w & 1) : k);
+        const longlong2* ps = p + s * (3 * 32);
+        const longlong2* pq = p + fx_partner(w, s) * 32;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            o.s[k][c] = CG ? __ldcg(ps + c * 32) : __ldg(ps + c * 32);
+            o.q[k][c] = CG ? __ldcg(pq + c * 32) : __ldg(pq + c * 32);
+        }
+    }
+}
+
+template <int NS>
+__device__ __forceinline__ void fx_load_link(const StencilArgs& a, int w, int jl, FxOperands<NS>& o) {
+    const int4* L = a.fxl + fx_index(jl, 36) + (w >> 2) * (9 * 32);
+    if (w & 2) {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) o.u[k] = __ldg(L + k * 32);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) o.u[3 * (k % 3) + k / 3] = __ldg(L + k * 32);
+    }
+}
+
+// h (forward) or conj(h) (backward) of component c
+__device__ __forceinline__ void fx_project(int w, const longlong2 (&s)[3], const longlong2 (&q)[3], I2 (&h)[3]) {
+#define GS_FX_PROJECT(X, Y)                                              \
+    _Pragma("unroll") for (int c = 0; c < 3; ++c) h[c] = I2{X, Y};       \
+    break;
+    switch (w) {
+        case 0: case 1: case 8: GS_FX_PROJECT(s[c].x + q[c].y, s[c].y - q[c].x)        // s - i q
+        case 9: GS_FX_PROJECT(s[c].x - q[c].y, s[c].y + q[c].x)                        // s + i q
+        case 5: case 12: case 13: GS_FX_PROJECT(s[c].x - q[c].x, s[c].y - q[c].y)      // s - q
+        case 4: GS_FX_PROJECT(s[c].x + q[c].x, s[c].y + q[c].y)                        // s + q
+        case 2: case 3: case 10: GS_FX_PROJECT(s[c].x - q[c].y, -s[c].y - q[c].x)      // conj(s + i q)
+        case 11: GS_FX_PROJECT(s[c].x + q[c].y, q[c].x - s[c].y)                       // conj(s - i q)
+        case 6: GS_FX_PROJECT(s[c].x - q[c].x, q[c].y - s[c].y)                        // conj(s - q)
+        default: GS_FX_PROJECT(s[c].x + q[c].x, -s[c].y - q[c].y)                      // conj(s + q)
+    }
+#undef GS_FX_PROJECT
+}
+
+template <int NS>
+__device__ __forceinline__ void fx_hop(const FxOperands<NS>& o, int w, int sh, FxShared& sm, int lane) {
+    FxLimb hx[NS][3], hy[NS][3], hn[NS][3];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+        I2 h[3];
+        fx_project(w + k, o.s[k], o.q[k], h);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            hx[k][c] = fx_split(h[c].x);
+            hy[k][c] = fx_split(h[c].y);
+            hn[k][c] = fx_split(-h[c].y);
+        }
+    }
+    const long long half = sh > 0 ? 1ll << (sh - 1) : 0ll;
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+            FxAcc re = fx_start(half), im = fx_start(half);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const int4 u = o.u[3 * c + r];
+                const FxLimb ux{u.y, u.x}, uy{u.w, u.z};
+                fx_fma(re, ux, hx[k][c]);
+                fx_fma(re, uy, hn[k][c]);
+                fx_fma(im, ux, hy[k][c]);
+                fx_fma(im, uy, hx[k][c]);
+            }
+            sm.hop[w + k][lane][r] = make_longlong2(fx_take(re, sh), fx_take(im, sh));
+        }
+}
+
+// Epilogue dots of one complex output (see f64_tile).
+template <int EPI, bool CG>
+__device__ __forceinline__ void stencil_dots(const StencilArgs& a, int64_t i, double re, double im, double (&e)[5]) {
+    if (EPI == EPI_DOT_RHAT_V) {
+        const double2 rv = CG ? __ldcg(a.epi_vec + i) : a.epi_vec[i];
+        e[0] = fma(rv.x, re, fma(rv.y, im, e[0]));
+        e[1] = fma(rv.x, im, fma(-rv.y, re, e[1]));
+    } else if (EPI == EPI_DOT_TS || EPI == EPI_DOT_TSR) {
+        const double2 sv = CG ? __ldcg(a.epi_vec + i) : a.epi_vec[i];
+        e[0] = fma(re, sv.x, fma(im, sv.y, e[0]));
+        e[1] = fma(re, sv.y, fma(-im, sv.x, e[1]));
+        e[2] = fma(re, re, fma(im, im, e[2]));
+        if (EPI == EPI_DOT_TSR) {
+            const double2 rv = CG ? __ldcg(a.epi_vec2 + i) : a.epi_vec2[i];
+            e[3] = fma(rv.x, re, fma(rv.y, im, e[3]));
+            e[4] = fma(rv.x, im, fma(-rv.y, re, e[4]));
+        }
+    }
+}
+
+// The hops' contributions to one component of a site, spin = 0..3, colour c:
+// upper spins add g, lower spins X_mu^dag (g_back - g_fwd); backward rows hold
+// conj(g).
+__device__ __forceinline__ I2 fx_sum(const FxShared& sm, int site, int spin, int c) {
+    if (spin < 2) {
+        I2 t[4];
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu) {
+            const longlong2 f = sm.hop[4 * mu + spin][site][c], b = sm.hop[4 * mu + 2 + spin][site][c];
+            t[mu] = I2{f.x + b.x, f.y - b.y};
+        }
+        return (t[0] + t[1]) + (t[2] + t[3]);
+    }
+    const int s = spin - 2;
+    I2 d[4];
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+        const int w = 4 * mu + (mu < 2 ? 1 - s : s);
+        const longlong2 f = sm.hop[w][site][c], b = sm.hop[w + 2][site][c];
+        d[mu] = I2{b.x - f.x, -b.y - f.y};
+    }
+    if (s == 0) return fx_sub_i(fx_sub_i(d[1] + d[3], d[0]), d[2]);   // -i d0 + d1 - i d2 + d3
+    return fx_add_i(fx_sub_i(d[3] - d[1], d[0]), d[2]);               // -i d0 - d1 + i d2 + d3
+}
+
+// The label of the tile's site `lane`'s neighbour that hop w reads (-1: no such
+// site); fetched a tile ahead of its use.
+__device__ __forceinline__ int fx_label(const StencilArgs& a, int64_t base, int ts, int w) {
+    const int64_t k = base + (threadIdx.x & 31);
+    if ((int)(threadIdx.x & 31) >= ts || k >= a.n_out) return -1;
+    const int2 n = __ldg(a.nbr + (a.o0 + k) * 4 + (w >> 2));
+    return (w & 2) ? n.y : n.x;
+}
+
+// Exponent word of the input site with label l (kFxZero outside the input
+// range) and its index.
+template <bool CG>
+__device__ __forceinline__ int fx_site(const StencilArgs& a, int l, unsigned& i) {
+    i = l < 0 ? 0xffffffffu : (unsigned)l - (unsigned)a.a0;   // labels below the range wrap above it
+    if (i >= (unsigned)a.fxn) return kFxZero;
+    return CG ? __ldcg(a.fxe + i) : __ldg(a.fxe + i);
+}
+
+// One tile of ts <= 32 output sites from base, l = fx_label of this tile.
+// Phase 1: a warp per hop (and spin component).  Phase 2: three warps per spin
+// component, a thread one complex output: sum of the hops, conversion,
+// diagonal, addend and the epilogue dots.  Returns true, with nothing written,
+// if an input site of the tile does not fit fixed point.
+template <int EPI, bool CG, int NS>
+__device__ __forceinline__ bool fx_tile(const StencilArgs& a, int64_t base, int ts, int l, FxShared& sm,
+                                        int (&sE)[8][kSitesPerBlock], double (&e)[5]) {
+    const int warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    const int w = warp * NS;
+    bool bad;
+    {
+        unsigned i;
+        const int x = fx_site<CG>(a, l, i);
+        FxOperands<NS> o;
+        if (i < (unsigned)a.fxn) {
+            fx_load_spinor<NS, CG>(a, w, (int)i, o);
+            fx_load_link<NS>(a, w, (w & 2) ? l : (int)(a.o0 + base) + lane, o);
+        }
+        bad = x < 0;
+        if (NS == 2 || !(w & 1)) sE[w >> 1][lane] = x;
+        __syncthreads();
+        int E = 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) E = max(E, sE[q][lane]);
+        if (x > 0 && E - x < 63) {
+            fx_hop<NS>(o, w, E - x, sm, lane);
+        } else {
+#pragma unroll
+            for (int k = 0; k < NS; ++k)
+#pragma unroll
+                for (int q = 0; q < 3; ++q) sm.hop[w + k][lane][q] = make_longlong2(0, 0);
+        }
+    }
+    if (__syncthreads_or(bad)) return true;
+    for (int v = warp; v < 12; v += kFxThreads<NS> / 32) {
+        const int spin = v / 3;
+        const int i = (v - 3 * spin) * 32 + lane;
+        const int site = i / 3, c = i - 3 * site;
+        if (site >= ts || base + site >= a.n_out) continue;
+        const I2 t = fx_sum(sm, site, spin, c);
+        int E = 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) E = max(E, sE[q][site]);
+        const int64_t j = a.o0 + base + site;
+        const int k = 3 * spin + c;
+        const double2* self = nullptr;
+        if (j >= a.a0 && j < a.a1) self = a.inA + (j - a.a0) * kSiteC + k;
+        else if (j >= a.a1 && j < a.b1) self = a.inB + (j - a.a1) * kSiteC + k;
+        const int64_t o = (base + site) * kSiteC + k;
+        double re = fx_to_double(t.x, E), im = fx_to_double(t.y, E);
+        if (self) {
+            const double2 sv = CG ? __ldcg(self) : __ldg(self);
+            re = fma(a.diag, sv.x, re);
+            im = fma(a.diag, sv.y, im);
+        }
+        if (a.negate) {
+            re = -re;
+            im = -im;
+        }
+        if (a.addend) {
+            const double2 av = CG ? __ldcg(a.addend + o) : a.addend[o];
+            re += av.x;
+            im += av.y;
+        }
+        a.out[o] = make_double2(re, im);
+        stencil_dots<EPI, CG>(a, o, re, im, e);
+    }
+    __syncthreads();
+    return false;
+}
+
+// The block's tiles of the stencil; those that fixed point cannot hold (all of
+// them when a link does not fit) are done in double precision afterwards, so
+// that the rare path costs the common one no registers.
+template <int EPI, bool CG, int NS>
+__device__ __forceinline__ void fx_stencil(const StencilArgs& a, int ts, bool links_bad, FxShared& sm,
+                                           int (&sE)[8][kSitesPerBlock], int l, double (&e)[5]) {
+    const int64_t step = (int64_t)gridDim.x * ts;
+    const int w = (threadIdx.x >> 5) * NS;
+    bool any = links_bad;
+    if (!links_bad)
+        for (int64_t base = (int64_t)blockIdx.x * ts; base < a.n_out; base += step) {
+            const int next = fx_label(a, base + step, ts, w);
+            any |= fx_tile<EPI, CG, NS>(a, base, ts, l, sm, sE, e);
+            l = next;
+        }
+    if (any)
+        for (int64_t base = (int64_t)blockIdx.x * ts; base < a.n_out; base += step) {
+            unsigned i;
+            const bool bad = fx_site<CG>(a, fx_label(a, base, ts, w), i) < 0;
+            if (__syncthreads_or(bad) || links_bad) f64_tile<EPI, CG>(a, base, ts, sm.f64, e);
+        }
+}
+
+}  // namespace
+}  // namespace gs

@@ -115,6 +115,8 @@ struct Plan {
     int32_t* label = nullptr;    // [V] site -> label
     int2* nbr = nullptr;         // [V][4] (fwd label, bwd label) per mu, label-indexed
     double2* links = nullptr;    // [V][4][9] -1/2 U_mu(perm[j]) in label order
+    int4* fx_links = nullptr;    // the same in fixed point (fx.cuh): limbs (re.lo, re.hi, im.lo, im.hi)
+    int* fx_flag = nullptr;      // device: 1 if a link lies outside fixed point's range
     bool links_ready = false;
     long long hops[2][2] = {{0, 0}, {0, 0}};  // [out set][in set] in-set neighbour terms (0 = b, 1 = r)
     double2* dtinv = nullptr;    // [V - nb][12][12] inverse block row sums of D_rr (Reusken), lazily
@@ -186,8 +188,7 @@ struct gs_ctx;
 
 namespace gs {
 // The blocks of the persistent solver kernels of one schur_solve_batched
-// call.  Those kernels all have 128 threads and the same registers, so their
-// blocks are interchangeable and the GPU holds per_sm x SMs of them at once.
+// call.  In one call those blocks all have one size, so they are interchangeable and the GPU holds per_sm x SMs of them at once.
 // held[] records, per running solve, the blocks its kernel may have in
 // flight: its last grid (its previous kernel has finished before it launches
 // again), or nothing before its first launch.  A grid is granted only from
@@ -200,6 +201,7 @@ struct BlockLedger {
     std::condition_variable cv;
     std::atomic<int> running{0};
     int64_t reserve = 1;
+    bool resident = false;   // every problem's FP64 inner solves fit the on-chip kernel (persistent_fx.cu)
     struct Entry {
         const gs_ctx* ctx;
         int64_t blocks;
@@ -209,10 +211,12 @@ struct BlockLedger {
 };
 void ledger_enter(BlockLedger* L, const gs_ctx* c);
 void ledger_leave(BlockLedger* L, const gs_ctx* c);
-// blocks for c's next cooperative grid: at most want and target, never more
-// than the others leave free; 0 if none became free within the context's
-// wait limit x 60
-int64_t ledger_grant(gs_ctx* c, int per_sm, int64_t want, int64_t target);
+// blocks for c's next cooperative grid out of `capacity`: at most want and
+// target, at least `least`, never more than the others leave free; 0 if they
+// did not become free within the context's wait limit x 60
+int64_t ledger_grant(gs_ctx* c, int64_t capacity, int64_t want, int64_t target, int64_t least = 1);
+// c's last grid has ended (the host has waited for it): its blocks are free
+void ledger_release(gs_ctx* c);
 }  // namespace gs
 
 struct gs_ctx {
@@ -226,6 +230,8 @@ struct gs_ctx {
     std::vector<gs::Plan*> plans;      // plans[0] = identity
     gs::InnerWork inner;
     gs::OuterWork outer;
+    longlong2* fx_m = nullptr;         // fixed-point copy of a stencil input (fx.cuh): mantissas
+    int* fx_e = nullptr;               // and exponents [sites]
     double2* full_a = nullptr;         // [V][12] label-ordered scratch
     double2* full_b = nullptr;
     double2* full_c = nullptr;
@@ -243,6 +249,7 @@ struct gs_ctx {
     unsigned long long wait_ns = 1000000000ull;  // bound on every device-side wait (GS_OPT_WAIT_LIMIT_US)
     int opt_coop_blocks = 0;           // blocks of this context's cooperative grids in a batched solve (0 = by share)
     void* persist = nullptr;           // persistent-solver scratch (persistent.cu)
+    void* persist_fx = nullptr;        // and of the fixed-point one (persistent_fx.cu)
     void* multi = nullptr;             // multi-RHS workspaces (multi.cu)
     int coop_block_cap = 0;            // cap on cooperative grids (0 = whole GPU; batched solves)
     // batched solves: the block ledger of the schur_solve_batched call this
@@ -340,8 +347,18 @@ struct StencilArgs {
     BicgState* st;
     RedScratch red;
     int* ran;                // profiling: set to 1 if the launch did work, 0 if it exited early
+    // fixed point (fx.cuh; filled by fx_args): the input's mantissas and
+    // exponents, indexed by label - a0 (fxn sites), and the plan's links
+    const longlong2* fxm;
+    const int* fxe;
+    int64_t fxn;
+    const int4* fxl;
+    const int* fxflag;
 };
 gs_status launch_stencil_f64(gs_ctx* c, const StencilArgs& a);
+// fills the fixed-point fields for plan p and an n-site input held at (m, e)
+void fx_args(const Plan* p, const longlong2* m, const int* e, int64_t n, StencilArgs* a);
+gs_status launch_stencil_fx(gs_ctx* c, const StencilArgs& a, int grid);
 gs_status launch_stencil_f64_on(const StencilArgs& a, cudaStream_t stream);
 // profiling (api.cu): work counted for one stencil launch on plan p
 void stencil_work(const gs_ctx* c, const Plan* p, const StencilArgs& a, long long* hops,
@@ -407,6 +424,10 @@ gs_status net_conv_tc(gs_ctx* c, const __nv_bfloat162* in, float2* out, const __
 gs_status inner_fgmres_net(gs_ctx* c, const Plan* p, const double2* r, double2* e, double tol,
                            int m, int* iters_out);
 void free_persist(gs_ctx* c);
+void free_persist_fx(gs_ctx* c);
+constexpr int kFxUnfit = 100;   // BicgState status: the problem does not fit fixed point, nothing was solved
+gs_status persistent_bicg_fx(gs_ctx* c, const Plan* p, const StencilArgs& S, const double2* b, double2* x,
+                             InnerWork& w, double tol, int maxit);
 gs_status persistent_bicg_f64(gs_ctx* c, const StencilArgs& A, const StencilArgs& C,
                               const double2* b, double2* x, InnerWork& w, int64_t n, double tol,
                               int maxit);

@@ -4,7 +4,7 @@
 // apply P and P^T to spinor fields.
 #include <stdarg.h>
 
-#include "gs_internal.cuh"
+#include "fx.cuh"
 
 namespace gs {
 
@@ -129,16 +129,34 @@ __global__ void k_count_hops(int64_t V, int64_t nb, const int2* __restrict__ nbr
         if (loc[q]) atomicAdd(hops + q, loc[q]);
 }
 
-// links[j][mu][k] = -1/2 * U[perm[j]][mu][k]  (the factor is exact in binary)
-__global__ void k_pack_links(int64_t V, const int32_t* __restrict__ perm,
-                             const double2* __restrict__ U, double2* __restrict__ links) {
-    const int64_t n = V * 36;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = i / 36;
-        const int k = (int)(i % 36);
-        const double2 u = U[(int64_t)perm[j] * 36 + k];
-        links[i] = make_double2(-0.5 * u.x, -0.5 * u.y);
+// links[j][mu][k] = -1/2 * U[perm[j]][mu][k]  (the factor is exact in binary),
+// and the same in fixed point, in groups of 32 labels (fx_index): a block turns
+// 32 sites around in shared memory so that both arrays are written in whole
+// lines.  *flag = 1 if an entry does not fit fixed point (the stencils then
+// use the double-precision links).
+__global__ void __launch_bounds__(256) k_pack_links(int64_t V, const int32_t* __restrict__ perm,
+                                                    const double2* __restrict__ U, double2* __restrict__ links,
+                                                    int4* __restrict__ fx, int* __restrict__ flag) {
+    __shared__ int4 sm[32][37];
+    for (int64_t base = (int64_t)blockIdx.x * 32; base < V; base += (int64_t)gridDim.x * 32) {
+        const int n = (int)(V - base < 32 ? V - base : 32);
+        for (int i = threadIdx.x; i < n * 36; i += 256) {
+            const int site = i / 36, k = i - site * 36;
+            const double2 u = U[(int64_t)perm[base + site] * 36 + k];
+            const double2 l = make_double2(-0.5 * u.x, -0.5 * u.y);
+            links[base * 36 + i] = l;
+            const bool fits = fabs(l.x) <= kFxLinkMax && fabs(l.y) <= kFxLinkMax;   // false for NaN
+            if (!fits) atomicExch(flag, 1);
+            const FxLimb re = fx_split(fits ? __double2ll_rn(l.x * 0x1p61) : 0);
+            const FxLimb im = fx_split(fits ? __double2ll_rn(l.y * 0x1p61) : 0);
+            sm[site][k] = make_int4(re.lo, re.hi, im.lo, im.hi);
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < 36 * 32; i += 256) {
+            const int k = i >> 5, site = i & 31;
+            if (site < n) fx[base * 36 + i] = sm[site][k];
+        }
+        __syncthreads();
     }
 }
 
@@ -178,15 +196,17 @@ void free_plan(Plan* p) {
     cudaFree(p->label);
     cudaFree(p->nbr);
     cudaFree(p->links);
+    cudaFree(p->fx_links);
+    cudaFree(p->fx_flag);
     cudaFree(p->dtinv);
     delete p;
 }
 
 gs_status pack_plan_links(gs_ctx* c, Plan* p) {
     if (!c->have_gauge) return GS_OK;
-    const int64_t n = c->V * 36;
-    k_pack_links<<<grid_for(n, 256, c->num_sms * 16), 256, 0, c->stream>>>(c->V, p->perm, c->U_abi,
-                                                                          p->links);
+    GS_CUDA(c, cudaMemsetAsync(p->fx_flag, 0, sizeof(int), c->stream));
+    k_pack_links<<<grid_for(c->V, 32, c->num_sms * 16), 256, 0, c->stream>>>(c->V, p->perm, c->U_abi, p->links,
+                                                                            p->fx_links, p->fx_flag);
     c->launches++;
     GS_CHECK_LAUNCH(c);
     p->links_ready = true;
@@ -225,7 +245,9 @@ gs_status get_plan(gs_ctx* c, int type, int dir, int inverse, Plan** out) {
     if (cudaMalloc(&p->perm, V * sizeof(int32_t)) != cudaSuccess ||
         cudaMalloc(&p->label, V * sizeof(int32_t)) != cudaSuccess ||
         cudaMalloc(&p->nbr, V * 4 * sizeof(int2)) != cudaSuccess ||
-        cudaMalloc(&p->links, V * 36 * sizeof(double2)) != cudaSuccess) {
+        cudaMalloc(&p->links, V * 36 * sizeof(double2)) != cudaSuccess ||
+        cudaMalloc(&p->fx_links, fx_padded(V) * 36 * sizeof(int4)) != cudaSuccess ||
+        cudaMalloc(&p->fx_flag, sizeof(int)) != cudaSuccess) {
         free_plan(p);
         cudaGetLastError();
         return set_err(c, GS_ENOMEM, "allocating a permutation plan for V = %lld failed",

@@ -680,7 +680,7 @@ static int coop_grid(gs_ctx* c, K kernel, int64_t want, int64_t rest_sites, int6
         const bool small = rest_sites <= kBatchMaxRestSites;
         const int64_t target = (small && round > 0) ? round
                                : (small && per_sm > 2 ? 2 : per_sm) * (int64_t)c->num_sms / n;
-        return (int)ledger_grant(c, per_sm, w, target > 0 ? target : 1);
+        return (int)ledger_grant(c, full, w, target > 0 ? target : 1);
     }
     int64_t g = coop_blocks(c, per_sm, rest_sites);
     if (want < g) g = want;

@@ -7,7 +7,7 @@
 #include <complex>
 #include <vector>
 
-#include "gs_internal.cuh"
+#include "fx.cuh"
 
 namespace gs {
 
@@ -58,7 +58,7 @@ gs_status ensure_inner(gs_ctx* c, int64_t sites) {
             cudaFree(*pp);
             *pp = nullptr;
         }
-        const size_t bytes = (size_t)sites * kSiteC * sizeof(double2);
+        const size_t bytes = (size_t)fx_padded(sites) * kSiteC * sizeof(double2);
         for (auto pp : v) {
             gs_status s = alloc_dev(c, (void**)pp, bytes);
             if (s != GS_OK) return s;
@@ -139,9 +139,6 @@ gs_status inner_solve_f64(gs_ctx* c, const Plan* p, const double2* t, double2* z
     gs_status s = ensure_inner(c, nr);
     if (s != GS_OK) return s;
     InnerWork& w = c->inner;
-    if (c->opt_inner_kernel != 0 && (s = launch_bicg_init(c, w, t, z, n, o.inner_tol)) != GS_OK)
-        return s;
-
     StencilArgs k1 = rr_args(c, p, w.v, w.p);
     k1.epi = EPI_DOT_RHAT_V;
     k1.epi_vec = w.rhat;
@@ -154,15 +151,30 @@ gs_status inner_solve_f64(gs_ctx* c, const Plan* p, const double2* t, double2* z
     k3.red = w.red;
 
     volatile BicgPublic* pub = w.pub_host;
-    if (c->opt_inner_kernel == 0) {
-        // the whole solve in one cooperative launch (persistent.cu)
+    int kernel = c->opt_inner_kernel;
+    if (kernel == 0) {
+        // the whole solve in one cooperative launch (persistent_fx.cu); a field
+        // or right-hand side that fixed point cannot hold goes to the
+        // double-precision kernel (persistent.cu), or inside a batched call,
+        // whose block ledger counts blocks of one size, to the per-phase launches
         int slot = -1;
         if (c->prof.on && (s = prof_begin(c, &slot)) != GS_OK) return s;
-        s = persistent_bicg_f64(c, k1, k3, t, z, w, n, o.inner_tol, o.inner_max_iter);
-        if (s != GS_OK) return s;
-        if (slot >= 0) GS_CUDA(c, cudaEventRecord(c->prof.ev[2 * slot + 1], c->stream));
-        GS_CUDA(c, cudaEventRecord(w.ev[0], c->stream));
-        GS_CUDA(c, cudaEventSynchronize(w.ev[0]));
+        auto finished = [&]() -> gs_status {
+            if (slot >= 0) GS_CUDA(c, cudaEventRecord(c->prof.ev[2 * slot + 1], c->stream));
+            GS_CUDA(c, cudaEventRecord(w.ev[0], c->stream));
+            GS_CUDA(c, cudaEventSynchronize(w.ev[0]));
+            return GS_OK;
+        };
+        s = persistent_bicg_fx(c, p, k1, t, z, w, o.inner_tol, o.inner_max_iter);
+        if (s != GS_OK || (s = finished()) != GS_OK) return s;
+        ledger_release(c);
+        if (pub->status == kFxUnfit) {
+            if (c->ledger) kernel = 1;
+            else {
+                s = persistent_bicg_f64(c, k1, k3, t, z, w, n, o.inner_tol, o.inner_max_iter);
+                if (s != GS_OK || (s = finished()) != GS_OK) return s;
+            }
+        }
         if (slot >= 0) {
             // algorithmic FP64 work: two D_rr applications per iteration and the
             // vector updates (84 flop per complex entry per iteration)
@@ -177,7 +189,9 @@ gs_status inner_solve_f64(gs_ctx* c, const Plan* p, const double2* t, double2* z
                 {slot, 3, (long long)(2 * it * nr), (long long)(2 * it * hops),
                  it * (2.0 * fl + 84.0 * (double)n), it * (2.0 * by + 14.0 * 16.0 * (double)n)});
         }
-    } else {
+    }
+    if (kernel != 0) {
+        if ((s = launch_bicg_init(c, w, t, z, n, o.inner_tol)) != GS_OK) return s;
         // Iterations are queued ahead of the GPU; the host waits on the event of
         // the iteration `depth` behind and reads the mapped `done` flag, so at most
         // `depth` no-op iterations are queued after convergence.
