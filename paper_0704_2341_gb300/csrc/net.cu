@@ -26,7 +26,7 @@
 #include <complex>
 #include <vector>
 
-#include "gs_internal.cuh"
+#include "warp_sum.cuh"
 
 struct gs_net {
     int C = 0;
@@ -343,6 +343,7 @@ __global__ void k_net_restrict64(const float2* __restrict__ full, const int32_t*
 // ---------------------------------------------------------------------------
 constexpr int kFgBlas = 256;
 constexpr int kFgChunk = 8;
+constexpr int kFgCounters = (kMaxRestart + 1 + kFgChunk - 1) / kFgChunk;   // one per chunk of vectors
 
 // v = s r (FP64 AoS rest vector -> FP32 layout)
 __global__ void k_fg_pack(const double2* __restrict__ r, float4* __restrict__ v, int64_t nr, double sc) {
@@ -384,18 +385,25 @@ __global__ void k_net_restrict_lp(const float2* __restrict__ full, const int32_t
         v[i] = make_float4(a.x, a.y, b.x, b.y);
     }
 }
-// out[k] = <X_k, y> (k < nvec), FP32 products summed per thread, FP64 across
-// threads and blocks; block (bx, chunk) takes vectors 8 chunk .. + 7 against
-// one load of y; the last block adds the per-block partials in block order
-__global__ void k_fg_multidot(const float2* __restrict__ X, int64_t ld, const float2* __restrict__ y, int64_t n,
-                              int nvec, double2* out, double* partial, unsigned int* counter) {
-    __shared__ double sm[kFgBlas / 32][2 * kFgChunk];
+// out[k] = <X_k, y> (k < nvec), FP32 products summed per thread, 64-bit sums
+// across threads and blocks; block (bx, chunk) takes vectors 8 chunk .. + 7
+// against one load of y; a chunk's last block adds its per-block partials.
+// HBM bound: (nvec + 1) n x 8 bytes.  The sums across threads were FP64 shuffles
+// and one thread per vector added 1216 partials: 190 us a call on 16^3 x 32 (mean
+// over a cycle of FGMRES), of which the vectors' bytes are 26; through shared
+// memory and integer warp sums 33.
+__global__ void __launch_bounds__(kFgBlas) k_fg_multidot(const float2* __restrict__ X, int64_t ld,
+                                                         const float2* __restrict__ y, int64_t n, int nvec,
+                                                         double2* out, double* partial, unsigned int* counter) {
+    constexpr int V2 = 2 * kFgChunk;
+    __shared__ float sm[V2][kFgBlas];
     __shared__ bool am_last;
     const int k0 = blockIdx.y * kFgChunk;
     const int nk = nvec - k0 < kFgChunk ? nvec - k0 : kFgChunk;
-    float a[2 * kFgChunk];
+    float a[V2];
 #pragma unroll
-    for (int q = 0; q < 2 * kFgChunk; ++q) a[q] = 0.f;
+    for (int q = 0; q < V2; ++q) a[q] = 0.f;
+#pragma unroll 2
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float2 w = y[i];
 #pragma unroll
@@ -407,44 +415,41 @@ __global__ void k_fg_multidot(const float2* __restrict__ X, int64_t ld, const fl
             }
         }
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int NW = kFgBlas / 32;
 #pragma unroll
-    for (int q = 0; q < 2 * kFgChunk; ++q) {
-        double v = (double)a[q];
+    for (int q = 0; q < V2; ++q) sm[q][threadIdx.x] = a[q];
+    __syncthreads();
+    double* part = partial + (int64_t)k0 * gridDim.x * 2;      // [vector of the chunk][re, im][block]
+    for (int q = warp; q < 2 * nk; q += NW) {
+        float x[NW];
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (lane == 0) sm[warp][q] = v;
+        for (int m = 0; m < NW; ++m) x[m] = sm[q][m * 32 + lane];
+        const double t = warp_sum<NW>(x);
+        if (lane == 0) part[(int64_t)q * gridDim.x + blockIdx.x] = t;
     }
     __syncthreads();
-    const unsigned nblocks = gridDim.x * gridDim.y;
     if (threadIdx.x == 0) {
-        for (int q = 0; q < nk; ++q) {
-            double s0 = 0.0, s1 = 0.0;
-            for (int w = 0; w < nw; ++w) {
-                s0 += sm[w][2 * q];
-                s1 += sm[w][2 * q + 1];
-            }
-            double* part = partial + ((int64_t)(k0 + q) * gridDim.x + blockIdx.x) * 2;
-            part[0] = s0;
-            part[1] = s1;
-        }
         __threadfence();
-        am_last = atomicAdd(counter, 1u) == nblocks - 1;
+        am_last = atomicAdd(counter + blockIdx.y, 1u) == gridDim.x - 1;
     }
     __syncthreads();
     if (!am_last) return;
     __threadfence();
-    for (int kk = threadIdx.x; kk < nvec; kk += blockDim.x) {
-        double s0 = 0.0, s1 = 0.0;
-        const double* part = partial + (int64_t)kk * gridDim.x * 2;
-#pragma unroll 8
-        for (unsigned b = 0; b < gridDim.x; ++b) {
-            s0 += __ldcg(part + 2 * b);
-            s1 += __ldcg(part + 2 * b + 1);
+    for (int q = warp; q < 2 * nk; q += NW) {
+        double t = 0.0;
+        for (unsigned b0 = 0; b0 < gridDim.x; b0 += 32 * 10) {
+            double x[10];
+#pragma unroll
+            for (int m = 0; m < 10; ++m) {
+                const unsigned b = b0 + 32 * m + lane;
+                x[m] = b < gridDim.x ? __ldcg(part + (int64_t)q * gridDim.x + b) : 0.0;
+            }
+            t += warp_sum<10>(x);
         }
-        out[kk] = make_double2(s0, s1);
+        if (lane == 0) ((double*)out)[2 * k0 + q] = t;
     }
-    if (threadIdx.x == 0) *counter = 0u;
+    if (threadIdx.x == 0) counter[blockIdx.y] = 0u;
 }
 // y += sign sum_k coef[k] X_k (coefficients FP64 on the device)
 __global__ void k_fg_multiaxpy(const float2* __restrict__ X, int64_t ld, int nvec, const double2* __restrict__ coef,
@@ -724,8 +729,9 @@ gs_status net_apply_rest(gs_ctx* c, gs_net* nt, const Plan* p, const double2* t,
 static gs_status fg_multidot(gs_ctx* c, const float2* X, int64_t ld, int nvec, const float2* y, int64_t n,
                              double2* out) {
     const int nchunks = (nvec + kFgChunk - 1) / kFgChunk;
+    // 8 blocks of 256 threads fill an SM; with more chunks than that each gets two blocks an SM
     int64_t cap = (int64_t)c->num_sms * 8 / nchunks;
-    if (cap < 64) cap = 64;
+    if (cap < 2 * c->num_sms) cap = 2 * c->num_sms;
     if (cap > kRedScratchDoubles / (2 * nvec)) cap = kRedScratchDoubles / (2 * nvec);
     dim3 g(grid_for(n, kFgBlas, (int)cap), nchunks);
     k_fg_multidot<<<g, kFgBlas, 0, c->stream>>>(X, ld, y, n, nvec, out, c->fg_red.partial, c->fg_red.counter);
@@ -802,11 +808,11 @@ gs_status inner_fgmres_net(gs_ctx* c, const Plan* p, const double2* r, double2* 
             cudaMalloc(&c->fg_y, (kMaxRestart + 1) * sizeof(double2)) != cudaSuccess ||
             cudaHostAlloc(&c->fg_y_host, (kMaxRestart + 1) * sizeof(double2), 0) != cudaSuccess ||
             cudaMalloc(&c->fg_red.partial, kRedScratchDoubles * sizeof(double)) != cudaSuccess ||
-            cudaMalloc(&c->fg_red.counter, sizeof(unsigned int)) != cudaSuccess) {
+            cudaMalloc(&c->fg_red.counter, kFgCounters * sizeof(unsigned int)) != cudaSuccess) {
             cudaGetLastError();
             return set_err(c, GS_ENOMEM, "allocating FGMRES scratch failed");
         }
-        GS_CUDA(c, cudaMemsetAsync(c->fg_red.counter, 0, sizeof(unsigned int), c->stream));
+        GS_CUDA(c, cudaMemsetAsync(c->fg_red.counter, 0, kFgCounters * sizeof(unsigned int), c->stream));
     }
     gs_status s;
     float2* V = c->fg_V;

@@ -27,6 +27,7 @@
 //     update of x and the norms run beside the hops' integer work.
 #include "dslash_fx.cuh"
 #include "gridsync.cuh"
+#include "warp_sum.cuh"
 
 namespace gs {
 namespace {
@@ -103,36 +104,6 @@ __device__ __noinline__ bool fx_still(const PArgsFx& P, unsigned long long& t0, 
     if (now - t0 <= P.wait_ns && spins <= (unsigned)kSpinLimit) return true;
     atomicExch(P.err, (int)GS_TIMEOUT);
     return false;
-}
-
-// The sum over the warp of N doubles per lane, in every lane.  Values are added
-// as 54-bit integers under the largest one's exponent (no two sums differ in
-// their order): the error is at most 2^-55 of the largest value per term, below
-// that of a double-precision tree, whose partial sums round at 2^-53.  Sums out
-// of the usual range take that tree.
-template <int N>
-__device__ __forceinline__ double warp_sum(const double (&x)[N]) {
-    int E = 0;
-#pragma unroll
-    for (int k = 0; k < N; ++k) E = max(E, fx_exponent((unsigned)__double2hiint(x[k])));
-    E = __reduce_max_sync(0xffffffffu, E);
-    if (E == 0) return 0.0;
-    if (E < kFxMinExp || E > 1900) {
-        double s = 0.0;
-#pragma unroll
-        for (int k = 0; k < N; ++k) s += x[k];
-#pragma unroll 1
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        return s;
-    }
-    long long m = 0;               // |term| <= 2^54, at most 16 terms
-#pragma unroll
-    for (int k = 0; k < N; ++k)
-        m += fx_from_bits((unsigned)__double2hiint(x[k]), (unsigned)__double2loint(x[k]), E + 6);
-    const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)m & 0x1fffffu);
-    const unsigned mid = __reduce_add_sync(0xffffffffu, (unsigned)(m >> 21) & 0x1fffffu);
-    const int hi = __reduce_add_sync(0xffffffffu, (int)(m >> 42));
-    return fx_to_double((long long)lo + ((long long)mid << 21) + ((long long)hi << 42), E + 3);
 }
 
 // Grid barrier and sums in one: tot = the sums over all threads of the grid of
