@@ -24,6 +24,7 @@
 #include <math.h>
 
 #include <complex>
+#include <type_traits>
 #include <vector>
 
 #include "warp_sum.cuh"
@@ -40,6 +41,7 @@ struct gs_net {
     long long step = 0;
     // scratch sized for a lattice
     int64_t capV = 0;
+    int capB = 0;            // samples the activations hold
     float2* act[4] = {};     // act0 [V][4][3], act1/2 [V][4C][3], act3 [V][4][3]
     float2* gact[2] = {};    // gradient buffers [V][4C][3]
     float2* partial = nullptr;  // [chunks][9][K][R]
@@ -62,6 +64,9 @@ namespace {
 constexpr int kTS = 8;           // sites per tile
 constexpr int kNCol = kTS * 3;   // GEMM columns per tile
 constexpr int kChunks = 32;      // site chunks of the weight gradient
+constexpr int kGroup = 4;        // samples of a training step that share each launch (24 channels)
+constexpr int kThinChunks = 304; // site chunks of the thin layers' weight gradients, over the group
+constexpr int kLossRed = 2 + 2 * 1024;   // floats of the loss reduction per sample
 
 __device__ __forceinline__ float2 cm(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -84,6 +89,54 @@ __device__ __forceinline__ float2 loadw(const __nv_bfloat162* W, int64_t i) {
     return __bfloat1622float2(W[i]);
 }
 
+// (U_d(x) in(x + d))[k, :] for one row k of a K-row field
+template <int K>
+__device__ __forceinline__ void transport_row(const float2* __restrict__ in, const float2* __restrict__ U32,
+                                              const int2* __restrict__ nbr, int64_t x, int d, int k, float2 (&t)[3]) {
+    int64_t y = x;
+    const float2* u = nullptr;
+    bool dag = false;
+    if (d >= 1 && d <= 4) {
+        const int mu = d - 1;
+        y = __ldg(nbr + x * 4 + mu).x;
+        u = U32 + (x * 4 + mu) * 9;
+    } else if (d >= 5) {
+        const int mu = d - 5;
+        y = __ldg(nbr + x * 4 + mu).y;
+        u = U32 + (y * 4 + mu) * 9;
+        dag = true;
+    }
+    const float2* src = in + (y * K + k) * 3;
+    const float2 p0 = src[0], p1 = src[1], p2 = src[2];
+    if (!u) {
+        t[0] = p0;
+        t[1] = p1;
+        t[2] = p2;
+        return;
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        float2 c0, c1, c2;
+        if (!dag) {
+            c0 = __ldg(u + 3 * a);
+            c1 = __ldg(u + 3 * a + 1);
+            c2 = __ldg(u + 3 * a + 2);
+        } else {  // U^dag: row a = conj of column a
+            c0 = __ldg(u + a);
+            c1 = __ldg(u + 3 + a);
+            c2 = __ldg(u + 6 + a);
+            c0.y = -c0.y;
+            c1.y = -c1.y;
+            c2.y = -c2.y;
+        }
+        float2 r = make_float2(0.f, 0.f);
+        cfma2(r, c0, p0);
+        cfma2(r, c1, p1);
+        cfma2(r, c2, p2);
+        t[a] = r;
+    }
+}
+
 // transported activations of one tile for transport d:
 // T[k][s*3 + a] = (U_d(x_s) in(x_s + d))[k, a]; threads stride over (s, k)
 template <int K>
@@ -92,56 +145,10 @@ __device__ __forceinline__ void stage_tile(const float2* __restrict__ in, const 
                                            float2 (*T)[kNCol]) {
     for (int e = threadIdx.x; e < kTS * K; e += blockDim.x) {
         const int s = e / K, k = e - s * K;
-        const int64_t x = base + s;
-        float2 t0 = make_float2(0.f, 0.f), t1 = t0, t2 = t0;
-        if (x < V) {
-            int64_t y = x;
-            const float2* u = nullptr;
-            bool dag = false;
-            if (d >= 1 && d <= 4) {
-                const int mu = d - 1;
-                y = __ldg(nbr + x * 4 + mu).x;
-                u = U32 + (x * 4 + mu) * 9;
-            } else if (d >= 5) {
-                const int mu = d - 5;
-                y = __ldg(nbr + x * 4 + mu).y;
-                u = U32 + (y * 4 + mu) * 9;
-                dag = true;
-            }
-            const float2* src = in + (y * K + k) * 3;
-            const float2 p0 = src[0], p1 = src[1], p2 = src[2];
-            if (!u) {
-                t0 = p0;
-                t1 = p1;
-                t2 = p2;
-            } else if (!dag) {
-                float2 r[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        float2 t[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        if (base + s < V) transport_row<K>(in, U32, nbr, base + s, d, k, t);
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    cfma2(r[a], __ldg(u + 3 * a + 0), p0);
-                    cfma2(r[a], __ldg(u + 3 * a + 1), p1);
-                    cfma2(r[a], __ldg(u + 3 * a + 2), p2);
-                }
-                t0 = r[0];
-                t1 = r[1];
-                t2 = r[2];
-            } else {  // U^dag: row a = conj of column a
-                float2 r[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const float2 c0 = __ldg(u + 0 + a), c1 = __ldg(u + 3 + a), c2 = __ldg(u + 6 + a);
-                    cfma2(r[a], make_float2(c0.x, -c0.y), p0);
-                    cfma2(r[a], make_float2(c1.x, -c1.y), p1);
-                    cfma2(r[a], make_float2(c2.x, -c2.y), p2);
-                }
-                t0 = r[0];
-                t1 = r[1];
-                t2 = r[2];
-            }
-        }
-        T[k][s * 3 + 0] = t0;
-        T[k][s * 3 + 1] = t1;
-        T[k][s * 3 + 2] = t2;
+        for (int a = 0; a < 3; ++a) T[k][s * 3 + a] = t[a];
     }
 }
 
@@ -150,6 +157,8 @@ template <int CIN, int COUT, class WT>
 __global__ void k_net_conv(const float2* __restrict__ in, float2* __restrict__ out, const WT* __restrict__ W,
                            const float2* __restrict__ U32, const int2* __restrict__ nbr, int64_t V) {
     constexpr int K = 4 * CIN, R4 = 4 * COUT;
+    in += (int64_t)blockIdx.y * V * K * 3;       // sample
+    out += (int64_t)blockIdx.y * V * R4 * 3;
     __shared__ float2 T[K][kNCol];
     const int R = threadIdx.x;
     for (int64_t base = (int64_t)blockIdx.x * kTS; base < V; base += (int64_t)gridDim.x * kTS) {
@@ -190,6 +199,8 @@ __global__ void k_net_conv(const float2* __restrict__ in, float2* __restrict__ o
 // out(x)[R, a] = sum_d (U_d(x) Phi_d(x + d)[R])[a]; one thread per (site, R)
 __global__ void k_net_phi_gather(const float2* __restrict__ phi, float2* __restrict__ out,
                                  const float2* __restrict__ U32, const int2* __restrict__ nbr, int64_t V) {
+    phi += (int64_t)blockIdx.y * V * 108;       // sample
+    out += (int64_t)blockIdx.y * V * 12;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < V * 4; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t x = i >> 2;
         const int R = (int)(i & 3);
@@ -275,16 +286,285 @@ __global__ void __launch_bounds__(256) k_net_gradw(const float2* __restrict__ in
     }
 }
 
-// G (+)= sum over chunks of the partials (fixed order)
-__global__ void k_net_reduce(const float2* __restrict__ partial, float2* __restrict__ G, int64_t nel,
-                             int chunks, int accumulate) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nel;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        float2 s = accumulate ? G[i] : make_float2(0.f, 0.f);
-        for (int c = 0; c < chunks; ++c) {
+// ---------------------------------------------------------------------------
+// The training kernels of the 24-channel network (FP32, one sample per grid row,
+// so that a group of samples shares each launch).  They replace one output
+// element per thread, whose operands came from shared memory at two loads per
+// complex multiply-add, by register tiles of 6 x 6: 12 loads for 36.
+// 8^4, per sample of a group of four: weight gradient of the C -> C layer 1082 ->
+// 185 us, its convolution 423 -> 204 us (FP32 floor at the measured 118
+// multiply-adds per clock per SM: 110 us each), C -> 1 convolution 305 -> 18 us,
+// thin weight gradients 76 -> 15 us; a step of four samples 9.3 -> 2.9 ms.
+// Packed multiply-adds help the convolution (226 -> 204 us: it shares its issue
+// slots with the weight loads) and not the weight gradient (185 -> 192 us).
+// ---------------------------------------------------------------------------
+constexpr int kC = 24, kRows = 4 * kC;      // channels, (channel, spin) rows
+constexpr int kPad = kRows + 2;             // row of a [column][row] tile: 16-byte aligned, conflict-free
+
+// (x, y) pairs for the packed multiply-add: one issue slot for two FP32
+// multiply-adds, each rounded as the scalar one is
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pk(float x, float y) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ void fma_f2(f2& a, f2 x, f2 y) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a) : "l"(x), "l"(y));
+}
+__device__ __forceinline__ float2 unpk(f2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+
+__device__ __forceinline__ void load6(const float2* p, float2 (&v)[6]) {
+    const float4* q = (const float4*)p;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const float4 x = q[i];
+        v[2 * i] = make_float2(x.x, x.y);
+        v[2 * i + 1] = make_float2(x.z, x.w);
+    }
+}
+
+// partial[chunk][d][k][R] of the C -> C layer: grid (chunks of a sample, 9, samples)
+__global__ void __launch_bounds__(256, 2) k_net_gradw24(const float2* __restrict__ in, const float2* __restrict__ gout,
+                                                       float2* __restrict__ partial, const float2* __restrict__ U32,
+                                                       const int2* __restrict__ nbr, int64_t V) {
+    __shared__ __align__(16) float2 T[kNCol][kPad], G[kNCol][kPad];
+    const int d = blockIdx.y;
+    const int64_t chunk = (int64_t)blockIdx.z * gridDim.x + blockIdx.x;
+    in += (int64_t)blockIdx.z * V * kRows * 3;
+    gout += (int64_t)blockIdx.z * V * kRows * 3;
+    const int64_t tiles = (V + kTS - 1) / kTS;
+    const int64_t t0 = tiles * blockIdx.x / gridDim.x, t1 = tiles * (blockIdx.x + 1) / gridDim.x;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;     // rows R = 6 tx .., k = 6 ty ..
+    float2 c[6][6] = {};
+    for (int64_t tile = t0; tile < t1; ++tile) {
+        const int64_t base = tile * kTS;
+        for (int e = threadIdx.x; e < kTS * kRows; e += 256) {
+            const int s = e / kRows, k = e - s * kRows;
+            float2 t[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+            if (base + s < V) transport_row<kRows>(in, U32, nbr, base + s, d, k, t);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) T[s * 3 + a][k] = t[a];
+        }
+        for (int e = threadIdx.x; e < kTS * kRows * 3; e += 256) {
+            const int s = e / (kRows * 3), q = e - s * (kRows * 3), R = q / 3, a = q - R * 3;
+            G[s * 3 + a][R] = base + s < V ? gout[(base + s) * (kRows * 3) + q] : make_float2(0.f, 0.f);
+        }
+        __syncthreads();
+#pragma unroll 2
+        for (int col = 0; col < kNCol; ++col) {
+            float2 g[6], t[6];
+            load6(&G[col][6 * tx], g);
+            load6(&T[col][6 * ty], t);
+#pragma unroll
+            for (int i = 0; i < 6; ++i)
+#pragma unroll
+                for (int j = 0; j < 6; ++j) cfmaconj(c[i][j], g[j], t[i]);
+        }
+        __syncthreads();
+    }
+    float2* dst = partial + (chunk * 9 + d) * (kRows * kRows);
+#pragma unroll
+    for (int i = 0; i < 6; ++i)
+#pragma unroll
+        for (int j = 0; j < 6; ++j) dst[(6 * ty + i) * kRows + 6 * tx + j] = c[i][j];
+}
+
+// out = sum_d W_d T_d of the C -> C layer: tiles of 16 sites (48 columns) by all
+// 96 rows, 128 threads; grid (tiles, samples)
+constexpr int kTS16 = 16, kCol16 = 48, kColPad = 50;
+__global__ void __launch_bounds__(128, 3) k_net_conv24(const float2* __restrict__ in, float2* __restrict__ out,
+                                                       const float2* __restrict__ W, const float2* __restrict__ U32,
+                                                       const int2* __restrict__ nbr, int64_t V) {
+    __shared__ __align__(16) float2 T[kRows][kColPad];
+    in += (int64_t)blockIdx.y * V * kRows * 3;
+    out += (int64_t)blockIdx.y * V * kRows * 3;
+    const int64_t base = (int64_t)blockIdx.x * kTS16;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;     // columns 6 ty .. (two sites); rows 2 tx + 32 j and
+    // the next, j = 0..2, so that a warp's weight loads are whole lines
+    f2 c[6][6] = {};
+    for (int d = 0; d < 9; ++d) {
+        for (int e = threadIdx.x; e < kTS16 * kRows; e += 128) {
+            const int s = e / kRows, k = e - s * kRows;
+            float2 t[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+            if (base + s < V) transport_row<kRows>(in, U32, nbr, base + s, d, k, t);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) T[k][s * 3 + a] = t[a];
+        }
+        __syncthreads();
+        const float2* wd = W + (int64_t)d * kRows * kRows + 2 * tx;
+#pragma unroll 4
+        for (int k = 0; k < kRows; ++k) {
+            float2 w[6], t[6];
+            const float4* wq = (const float4*)(wd + k * kRows);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const float4 x = __ldg(wq + 16 * i);
+                w[2 * i] = make_float2(x.x, x.y);
+                w[2 * i + 1] = make_float2(x.z, x.w);
+            }
+            load6(&T[k][6 * ty], t);
+            // acc += w t = w.x (t.x, t.y) + w.y (-t.y, t.x)
+            f2 t0[6], t1[6];
+#pragma unroll
+            for (int j = 0; j < 6; ++j) {
+                t0[j] = pk(t[j].x, t[j].y);
+                t1[j] = pk(-t[j].y, t[j].x);
+            }
+#pragma unroll
+            for (int i = 0; i < 6; ++i) {
+                const f2 w0 = pk(w[i].x, w[i].x), w1 = pk(w[i].y, w[i].y);
+#pragma unroll
+                for (int j = 0; j < 6; ++j) {
+                    fma_f2(c[i][j], w0, t0[j]);
+                    fma_f2(c[i][j], w1, t1[j]);
+                }
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int64_t x = base + 2 * ty + h;
+        if (x < V)
+#pragma unroll
+            for (int i = 0; i < 6; ++i)
+#pragma unroll
+                for (int a = 0; a < 3; ++a) out[(x * kRows + 2 * tx + 32 * (i >> 1) + (i & 1)) * 3 + a] = unpk(c[i][3 * h + a]);
+    }
+}
+
+// Phi[x][d][R] = W_d in(x) of the C -> 1 layer (W acts on channel and spin, U_d
+// on colour: the nine transports act on 4 rows afterwards, k_net_phi_gather,
+// instead of on 96 before); tiles of 8 sites, a thread 3 of the 36 rows (d, R) by
+// 2 columns; grid (tiles, samples)
+__global__ void __launch_bounds__(144) k_net_phi24(const float2* __restrict__ in, float2* __restrict__ phi,
+                                                   const float2* __restrict__ W, int64_t V) {
+    __shared__ __align__(16) float2 T[kRows][kNCol];
+    in += (int64_t)blockIdx.y * V * kRows * 3;
+    phi += (int64_t)blockIdx.y * V * 108;
+    const int64_t base = (int64_t)blockIdx.x * kTS;
+    for (int e = threadIdx.x; e < kTS * kRows * 3; e += 144) {
+        const int s = e / (kRows * 3), q = e - s * (kRows * 3), k = q / 3, a = q - k * 3;
+        T[k][s * 3 + a] = base + s < V ? in[(base + s) * (kRows * 3) + q] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    const int cg = threadIdx.x % 12, rg = threadIdx.x / 12;     // columns 2 cg .., rows 3 rg ..
+    float2 acc[3][2];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int k = 0; k < kRows; ++k) {
+        const float2 t0 = T[k][2 * cg], t1 = T[k][2 * cg + 1];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int row = 3 * rg + i, d = row >> 2, R = row & 3;
+            const float2 w = __ldg(W + ((int64_t)d * kRows + k) * 4 + R);
+            cfma2(acc[i][0], w, t0);
+            cfma2(acc[i][1], w, t1);
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+        const int col = 2 * cg + m, s = col / 3, a = col - s * 3;
+        if (base + s < V)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) phi[((base + s) * 36 + 3 * rg + i) * 3 + a] = acc[i][m];
+    }
+}
+
+// Weight gradients of the thin layers (FIRST: 1 -> C, else C -> 1) for all nine
+// transports in one pass over the 96-row field B: the 4-row field A is the one
+// that is transported.  1 -> C: A_d = T_d(in), B = gout, g_W[k, R] = B[R]
+// conj(A_d[k]).  C -> 1: U_d(x) in(x + d) against g(x) is in(y) against
+// U_d(x)^dag g(x), y = x + d, so A_d(y) = T of the reversed transport of gout,
+// B = in, g_W[k, R] = A_d[R] conj(B[k]).  192 threads: 6 of the 36 rows (d, .) by
+// 3 of the 96; partial[chunk][d][k][R]; grid (chunks of a sample, 1, samples).
+template <bool FIRST>
+__global__ void __launch_bounds__(192) k_net_gradw_thin(const float2* __restrict__ A4, const float2* __restrict__ B96,
+                                                        float2* __restrict__ partial, const float2* __restrict__ U32,
+                                                        const int2* __restrict__ nbr, int64_t V) {
+    __shared__ __align__(16) float2 A[kNCol][36 + 2], B[kNCol][kPad];
+    const int64_t chunk = (int64_t)blockIdx.z * gridDim.x + blockIdx.x;
+    A4 += (int64_t)blockIdx.z * V * 12;
+    B96 += (int64_t)blockIdx.z * V * kRows * 3;
+    const int64_t tiles = (V + kTS - 1) / kTS;
+    const int64_t t0 = tiles * blockIdx.x / gridDim.x, t1 = tiles * (blockIdx.x + 1) / gridDim.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;     // rows 6 warp .. of A; lane + 32 j of B
+    float2 acc[6][3];
+#pragma unroll
+    for (int i = 0; i < 6; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) acc[i][j] = make_float2(0.f, 0.f);
+    for (int64_t tile = t0; tile < t1; ++tile) {
+        const int64_t base = tile * kTS;
+        for (int e = threadIdx.x; e < kTS * 36; e += 192) {
+            const int s = e / 36, row = e - s * 36, d = row >> 2, r = row & 3;
+            const int dd = (FIRST || d == 0) ? d : (d <= 4 ? d + 4 : d - 4);
+            float2 t[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+            if (base + s < V) transport_row<4>(A4, U32, nbr, base + s, dd, r, t);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) A[s * 3 + a][row] = t[a];
+        }
+        for (int e = threadIdx.x; e < kTS * kRows * 3; e += 192) {
+            const int s = e / (kRows * 3), q = e - s * (kRows * 3), R = q / 3, a = q - R * 3;
+            B[s * 3 + a][R] = base + s < V ? B96[(base + s) * (kRows * 3) + q] : make_float2(0.f, 0.f);
+        }
+        __syncthreads();
+#pragma unroll 2
+        for (int col = 0; col < kNCol; ++col) {
+            float2 x[6], y[3];
+            load6(&A[col][6 * warp], x);
+#pragma unroll
+            for (int j = 0; j < 3; ++j) y[j] = B[col][lane + 32 * j];
+#pragma unroll
+            for (int i = 0; i < 6; ++i)
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    if (FIRST) cfmaconj(acc[i][j], y[j], x[i]);
+                    else cfmaconj(acc[i][j], x[i], y[j]);
+                }
+        }
+        __syncthreads();
+    }
+    float2* dst = partial + chunk * (9 * 4 * kRows);
+#pragma unroll
+    for (int i = 0; i < 6; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const int row = 6 * warp + i, d = row >> 2, r = row & 3, b = lane + 32 * j;
+            if (FIRST) dst[(d * 4 + r) * kRows + b] = acc[i][j];
+            else dst[(d * kRows + b) * 4 + r] = acc[i][j];
+        }
+}
+
+// G (+)= sum over chunks of the partials in a fixed order: 32 elements a block,
+// 8 threads an element
+__global__ void __launch_bounds__(256) k_net_reduce(const float2* __restrict__ partial, float2* __restrict__ G,
+                                                    int64_t nel, int chunks, int accumulate) {
+    __shared__ float2 sm[8][32];
+    const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
+    const int64_t i = blockIdx.x * (int64_t)32 + lane;
+    float2 s = make_float2(0.f, 0.f);
+    if (i < nel)
+#pragma unroll 4
+        for (int c = part; c < chunks; c += 8) {
             const float2 p = partial[(int64_t)c * nel + i];
             s.x += p.x;
             s.y += p.y;
+        }
+    sm[part][lane] = s;
+    __syncthreads();
+    if (part == 0 && i < nel) {
+        s = accumulate ? G[i] : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            s.x += sm[q][lane].x;
+            s.y += sm[q][lane].y;
         }
         G[i] = s;
     }
@@ -318,6 +598,8 @@ __global__ void k_net_embed64(const double2* __restrict__ t, const int32_t* __re
 }
 __global__ void k_net_embed32(const float2* __restrict__ t, const int32_t* __restrict__ perm, int64_t nb,
                               int64_t nr, float2* __restrict__ full) {
+    t += (int64_t)blockIdx.y * nr * 12;          // sample
+    full += (int64_t)blockIdx.y * (nb + nr) * 12;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nr * 12;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t k = i / 12;
@@ -482,6 +764,10 @@ __global__ void k_fg_scale(const float2* __restrict__ x, float2* __restrict__ y,
 __global__ void k_net_loss(const float2* __restrict__ yfull, const float2* __restrict__ z,
                            const int32_t* __restrict__ perm, int64_t nb, int64_t nr, float* red,
                            unsigned int* counter) {
+    yfull += (int64_t)blockIdx.y * (nb + nr) * 12;   // sample
+    z += (int64_t)blockIdx.y * nr * 12;
+    red += (int64_t)blockIdx.y * kLossRed;
+    counter += blockIdx.y;
     __shared__ float sm[2][32];
     __shared__ bool last;
     float a = 0.f, b = 0.f;
@@ -534,6 +820,10 @@ __global__ void k_net_loss(const float2* __restrict__ yfull, const float2* __res
 __global__ void k_net_lossgrad(const float2* __restrict__ yfull, const float2* __restrict__ z,
                                const int32_t* __restrict__ perm, int64_t nb, int64_t nr,
                                const float* __restrict__ red, float scale, float2* __restrict__ gfull) {
+    yfull += (int64_t)blockIdx.y * (nb + nr) * 12;   // sample
+    z += (int64_t)blockIdx.y * nr * 12;
+    gfull += (int64_t)blockIdx.y * (nb + nr) * 12;
+    red += (int64_t)blockIdx.y * kLossRed;
     const float coef = 2.f * scale / red[1];
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nr * 12;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -609,7 +899,10 @@ static void conv_dispatch(int C, int cin, int cout, const float2* in, float2* ou
         case 2: conv_dispatch_t<2, WT>(cin, cout, in, out, W, U32, nbr, V, blocks, s); break;
         case 4: conv_dispatch_t<4, WT>(cin, cout, in, out, W, U32, nbr, V, blocks, s); break;
         case 8: conv_dispatch_t<8, WT>(cin, cout, in, out, W, U32, nbr, V, blocks, s); break;
-        default: conv_dispatch_t<24, WT>(cin, cout, in, out, W, U32, nbr, V, blocks, s); break;
+        default:   // 24 channels in FP32: train_group
+            if constexpr (std::is_same<WT, __nv_bfloat162>::value)
+                conv_dispatch_t<24, WT>(cin, cout, in, out, W, U32, nbr, V, blocks, s);
+            break;
     }
 }
 
@@ -620,30 +913,32 @@ static void gradw_dispatch(int C, int cin, int cout, const float2* in, const flo
         case 2: gradw_dispatch_t<2>(cin, cout, in, gout, partial, U32, nbr, V, s); break;
         case 4: gradw_dispatch_t<4>(cin, cout, in, gout, partial, U32, nbr, V, s); break;
         case 8: gradw_dispatch_t<8>(cin, cout, in, gout, partial, U32, nbr, V, s); break;
-        default: gradw_dispatch_t<24>(cin, cout, in, gout, partial, U32, nbr, V, s); break;
+        default: break;   // 24 channels: train_group
     }
 }
 
 // scratch of a network for a lattice of V sites; FP32 links of the context
-static gs_status net_prepare(gs_ctx* c, gs_net* nt) {
+static gs_status net_prepare(gs_ctx* c, gs_net* nt, int B = 1) {
     const int64_t V = c->V;
-    if (nt->capV < V) {
+    if (nt->capV < V || nt->capB < B) {
         for (auto& a : nt->act) cudaFree(a);
         for (auto& a : nt->gact) cudaFree(a);
         cudaFree(nt->U32);
         nt->U32 = nullptr;
         nt->U32_src = nullptr;
-        const size_t big = (size_t)V * 4 * nt->C * 3 * sizeof(float2);
-        const size_t sm = (size_t)V * 12 * sizeof(float2);
+        const size_t big = (size_t)B * V * 4 * nt->C * 3 * sizeof(float2);
+        const size_t sm = (size_t)B * V * 12 * sizeof(float2);
         if (cudaMalloc(&nt->act[0], sm) != cudaSuccess || cudaMalloc(&nt->act[1], big) != cudaSuccess ||
             cudaMalloc(&nt->act[2], big) != cudaSuccess || cudaMalloc(&nt->act[3], sm) != cudaSuccess ||
             cudaMalloc(&nt->gact[0], big) != cudaSuccess || cudaMalloc(&nt->gact[1], big) != cudaSuccess ||
             cudaMalloc(&nt->U32, (size_t)V * 36 * sizeof(float2)) != cudaSuccess) {
             cudaGetLastError();
             nt->capV = 0;
+            nt->capB = 0;
             return set_err(c, GS_ENOMEM, "allocating network activations failed");
         }
         nt->capV = V;
+        nt->capB = B;
     }
     if (nt->U32_src != (const void*)c || !c->net_links_fresh) {
         k_links32<<<grid_for(V * 36, 256, c->num_sms * 8), 256, 0, c->stream>>>(c->U_abi, nt->U32, V * 36);
@@ -705,6 +1000,57 @@ static gs_status net_forward(gs_ctx* c, gs_net* nt, bool bf16) {
         c->launches++;
         GS_CHECK_LAUNCH(c);
     }
+    return GS_OK;
+}
+
+// Forward, loss and backward of n samples at once (24 channels, FP32 weights):
+// adds to (or with accumulate == 0 sets) the gradients of scale * sum of the
+// samples' losses, whose sums land in host_red.  Synchronises the stream.
+static gs_status train_group(gs_ctx* c, gs_net* nt, const Plan* p, const float2* t, const float2* z, int n, float scale,
+                             int accumulate) {
+    const Plan* id = c->plans[0];
+    const int64_t V = c->V, nb = p->nb, nr = V - nb;
+    const unsigned un = (unsigned)n;
+    const dim3 g(grid_for(nr * 12, 256, 1024), un), tiles((unsigned)((V + kTS - 1) / kTS), un),
+        tiles16((unsigned)((V + kTS16 - 1) / kTS16), un);
+    cudaStream_t st = c->stream;
+    auto reduce = [&](int l, int chunks) {
+        k_net_reduce<<<grid_for(nt->nel[l], 32, 1 << 30), 256, 0, st>>>(nt->partial, nt->G[l], nt->nel[l], chunks,
+                                                                      accumulate);
+    };
+    auto wprime = [&](int l, int K, int R4) {
+        k_net_wprime<<<grid_for(nt->nel[l], 256, 1024), 256, 0, st>>>(nt->W[l], nt->Wp, K, R4);
+    };
+    const size_t vec = (size_t)n * V * 12 * sizeof(float2);
+    GS_CUDA(c, cudaMemsetAsync(nt->act[0], 0, vec, st));
+    k_net_embed32<<<g, 256, 0, st>>>(t, p->perm, nb, nr, nt->act[0]);
+    // forward
+    k_net_conv<1, kC, float2><<<tiles, kRows, 0, st>>>(nt->act[0], nt->act[1], nt->W[0], nt->U32, id->nbr, V);
+    k_net_conv24<<<tiles16, 128, 0, st>>>(nt->act[1], nt->act[2], nt->W[1], nt->U32, id->nbr, V);
+    k_net_phi24<<<tiles, 144, 0, st>>>(nt->act[2], nt->gact[0], nt->W[2], V);
+    k_net_phi_gather<<<dim3(grid_for(V * 4, 256, c->num_sms * 8), un), 256, 0, st>>>(nt->gact[0], nt->act[3], nt->U32,
+                                                                                    id->nbr, V);
+    // loss and the gradient of the last activation (into gact[0], 12 per site)
+    k_net_loss<<<g, 256, 0, st>>>(nt->act[3], z, p->perm, nb, nr, nt->red, nt->counter);
+    GS_CUDA(c, cudaMemsetAsync(nt->gact[0], 0, vec, st));
+    k_net_lossgrad<<<g, 256, 0, st>>>(nt->act[3], z, p->perm, nb, nr, nt->red, scale, nt->gact[0]);
+    GS_CHECK_LAUNCH(c);
+    GS_CUDA(c, cudaMemcpyAsync(nt->host_red, nt->red, (size_t)n * kLossRed * sizeof(float), cudaMemcpyDeviceToHost, st));
+    // backward; a block of the weight gradients takes a chunk of one sample's sites
+    const unsigned thin = (unsigned)(kThinChunks / n), wide = (unsigned)(kChunks / n);
+    k_net_gradw_thin<false><<<dim3(thin, 1, un), 192, 0, st>>>(nt->gact[0], nt->act[2], nt->partial, nt->U32, id->nbr, V);
+    reduce(2, (int)thin * n);
+    wprime(2, kRows, 4);
+    k_net_conv<1, kC, float2><<<tiles, kRows, 0, st>>>(nt->gact[0], nt->gact[1], nt->Wp, nt->U32, id->nbr, V);
+    k_net_gradw24<<<dim3(wide, 9, un), 256, 0, st>>>(nt->act[1], nt->gact[1], nt->partial, nt->U32, id->nbr, V);
+    reduce(1, (int)wide * n);
+    wprime(1, kRows, kRows);
+    k_net_conv24<<<tiles16, 128, 0, st>>>(nt->gact[1], nt->gact[0], nt->Wp, nt->U32, id->nbr, V);
+    k_net_gradw_thin<true><<<dim3(thin, 1, un), 192, 0, st>>>(nt->act[0], nt->gact[0], nt->partial, nt->U32, id->nbr, V);
+    reduce(0, (int)thin * n);
+    GS_CHECK_LAUNCH(c);
+    c->launches += 16;
+    GS_CUDA(c, cudaStreamSynchronize(st));
     return GS_OK;
 }
 
@@ -944,9 +1290,9 @@ gs_status gs_net_create(gs_net** out, int channels) {
     const int64_t big = 9LL * 4 * channels * 4 * channels;
     ok = ok && cudaMalloc(&nt->Wp, big * sizeof(float2)) == cudaSuccess &&
          cudaMalloc(&nt->partial, (size_t)kChunks * big * sizeof(float2)) == cudaSuccess &&
-         cudaMalloc(&nt->red, 4096 * sizeof(float)) == cudaSuccess &&
-         cudaMalloc(&nt->counter, sizeof(unsigned int)) == cudaSuccess &&
-         cudaHostAlloc(&nt->host_red, 4 * sizeof(float), 0) == cudaSuccess &&
+         cudaMalloc(&nt->red, kGroup * kLossRed * sizeof(float)) == cudaSuccess &&
+         cudaMalloc(&nt->counter, kGroup * sizeof(unsigned int)) == cudaSuccess &&
+         cudaHostAlloc(&nt->host_red, kGroup * kLossRed * sizeof(float), 0) == cudaSuccess &&
          cudaHostAlloc(&nt->tc_err, sizeof(int), cudaHostAllocMapped) == cudaSuccess &&
          cudaHostGetDevicePointer(&nt->tc_err_dev, nt->tc_err, 0) == cudaSuccess;
     if (ok) *nt->tc_err = 0;
@@ -954,7 +1300,7 @@ gs_status gs_net_create(gs_net** out, int channels) {
         ok = cudaMalloc(&nt->Btc, net_tc_weight_elems() * sizeof(__nv_bfloat16)) == cudaSuccess &&
              cudaMalloc(&nt->Bphi, net_phi_weight_elems() * sizeof(__nv_bfloat16)) == cudaSuccess &&
              cudaMalloc(&nt->Bl1, net_l1_weight_elems() * sizeof(__nv_bfloat16)) == cudaSuccess;
-    if (ok) ok = cudaMemset(nt->counter, 0, sizeof(unsigned int)) == cudaSuccess &&
+    if (ok) ok = cudaMemset(nt->counter, 0, kGroup * sizeof(unsigned int)) == cudaSuccess &&
                  cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -1062,7 +1408,13 @@ gs_status gs_net_train_step(gs_ctx* c, gs_net* nt, int type, int dir, int invers
     Plan* p = nullptr;
     gs_status s = get_plan(c, type, dir, inverse, &p);
     if (s != GS_OK) return s;
-    if ((s = net_prepare(c, nt)) != GS_OK) return s;
+    // as many samples at once as 16 GB of activations hold, at most kGroup
+    int B = 1;
+    if (nt->C == kC)
+        while (B < kGroup && B < batch && (int64_t)(B + 1) * c->V * 4 * kC * 3 * 8 * 4 <= ((int64_t)16 << 30)) ++B;
+    s = net_prepare(c, nt, B);
+    if (s == GS_ENOMEM && B > 1) s = net_prepare(c, nt, B = 1);
+    if (s != GS_OK) return s;
     const Plan* id = c->plans[0];
     const int64_t V = c->V, nb = p->nb, nr = V - nb;
     const int g = grid_for(nr * 12, 256, 1024);
@@ -1070,45 +1422,57 @@ gs_status gs_net_train_step(gs_ctx* c, gs_net* nt, int type, int dir, int invers
     const float2* T = (const float2*)t_dev;
     const float2* Z = (const float2*)z_dev;
     double loss = 0.0;
-    for (int b = 0; b < batch; ++b) {
-        const float2* tb = T + (size_t)b * nr * 12;
-        const float2* zb = Z + (size_t)b * nr * 12;
-        GS_CUDA(c, cudaMemsetAsync(nt->act[0], 0, (size_t)V * 12 * sizeof(float2), c->stream));
-        k_net_embed32<<<g, 256, 0, c->stream>>>(tb, p->perm, nb, nr, nt->act[0]);
-        c->launches++;
-        if ((s = net_forward(c, nt, false)) != GS_OK) return s;
-        k_net_loss<<<g, 256, 0, c->stream>>>(nt->act[3], zb, p->perm, nb, nr, nt->red, nt->counter);
-        // gradient of the last activation into gact[0] (only 12 per site used)
-        GS_CUDA(c, cudaMemsetAsync(nt->gact[0], 0, (size_t)V * 12 * sizeof(float2), c->stream));
-        k_net_lossgrad<<<g, 256, 0, c->stream>>>(nt->act[3], zb, p->perm, nb, nr, nt->red,
-                                                 1.0f / batch, nt->gact[0]);
-        c->launches += 2;
-        GS_CUDA(c, cudaMemcpyAsync(nt->host_red, nt->red, 2 * sizeof(float), cudaMemcpyDeviceToHost,
-                                   c->stream));
-        // backward through the three layers
-        float2* gout = nt->gact[0];
-        float2* gin = nt->gact[1];
-        for (int l = 2; l >= 0; --l) {
-            int cin, cout;
-            layer_dims(nt->C, l, &cin, &cout);
-            gradw_dispatch(nt->C, cin, cout, nt->act[l], gout, nt->partial, nt->U32, id->nbr, V, c->stream);
-            k_net_reduce<<<grid_for(nt->nel[l], 256, 1024), 256, 0, c->stream>>>(nt->partial, nt->G[l],
-                                                                                 nt->nel[l], kChunks, b > 0);
-            c->launches += 2;
-            if (l > 0) {
-                k_net_wprime<<<grid_for(nt->nel[l], 256, 1024), 256, 0, c->stream>>>(nt->W[l], nt->Wp,
-                                                                                    4 * cin, 4 * cout);
-                conv_dispatch<float2>(nt->C, cout, cin, gout, gin, nt->Wp, nt->U32, id->nbr, V, blocks,
-                                      c->stream);
-                c->launches += 2;
-                float2* tmp = gout;
-                gout = gin;
-                gin = tmp;
-            }
-            GS_CHECK_LAUNCH(c);
+    if (nt->C == kC) {
+        // groups of samples share every launch
+        for (int b = 0; b < batch; b += B) {
+            const int n = batch - b < B ? batch - b : B;
+            if ((s = train_group(c, nt, p, T + (size_t)b * nr * 12, Z + (size_t)b * nr * 12, n, 1.0f / batch, b > 0)) !=
+                GS_OK)
+                return s;
+            for (int i = 0; i < n; ++i)
+                loss += (double)nt->host_red[i * kLossRed] / (double)nt->host_red[i * kLossRed + 1];
         }
-        GS_CUDA(c, cudaStreamSynchronize(c->stream));
-        loss += (double)nt->host_red[0] / (double)nt->host_red[1];
+    } else {
+        for (int b = 0; b < batch; ++b) {
+            const float2* tb = T + (size_t)b * nr * 12;
+            const float2* zb = Z + (size_t)b * nr * 12;
+            GS_CUDA(c, cudaMemsetAsync(nt->act[0], 0, (size_t)V * 12 * sizeof(float2), c->stream));
+            k_net_embed32<<<g, 256, 0, c->stream>>>(tb, p->perm, nb, nr, nt->act[0]);
+            c->launches++;
+            if ((s = net_forward(c, nt, false)) != GS_OK) return s;
+            k_net_loss<<<g, 256, 0, c->stream>>>(nt->act[3], zb, p->perm, nb, nr, nt->red, nt->counter);
+            // gradient of the last activation into gact[0] (only 12 per site used)
+            GS_CUDA(c, cudaMemsetAsync(nt->gact[0], 0, (size_t)V * 12 * sizeof(float2), c->stream));
+            k_net_lossgrad<<<g, 256, 0, c->stream>>>(nt->act[3], zb, p->perm, nb, nr, nt->red,
+                                                     1.0f / batch, nt->gact[0]);
+            c->launches += 2;
+            GS_CUDA(c, cudaMemcpyAsync(nt->host_red, nt->red, 2 * sizeof(float), cudaMemcpyDeviceToHost,
+                                       c->stream));
+            // backward through the three layers
+            float2* gout = nt->gact[0];
+            float2* gin = nt->gact[1];
+            for (int l = 2; l >= 0; --l) {
+                int cin, cout;
+                layer_dims(nt->C, l, &cin, &cout);
+                gradw_dispatch(nt->C, cin, cout, nt->act[l], gout, nt->partial, nt->U32, id->nbr, V, c->stream);
+                k_net_reduce<<<grid_for(nt->nel[l], 32, 1 << 30), 256, 0, c->stream>>>(nt->partial, nt->G[l],
+                                                                                     nt->nel[l], kChunks, b > 0);
+                c->launches += 2;
+                if (l > 0) {
+                    k_net_wprime<<<grid_for(nt->nel[l], 256, 1024), 256, 0, c->stream>>>(nt->W[l], nt->Wp,
+                                                                                        4 * cin, 4 * cout);
+                    conv_dispatch<float2>(nt->C, cout, cin, gout, gin, nt->Wp, nt->U32, id->nbr, V, blocks,
+                                          c->stream);
+                    c->launches += 2;
+                    float2* tmp = gout;
+                    gout = gin;
+                    gin = tmp;
+                }
+                GS_CHECK_LAUNCH(c);
+            }
+            GS_CUDA(c, cudaStreamSynchronize(c->stream));
+            loss += (double)nt->host_red[0] / (double)nt->host_red[1];
+        }
     }
     if (loss_out) *loss_out = (float)(loss / batch);
     if (update) {
