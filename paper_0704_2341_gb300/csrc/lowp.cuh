@@ -554,48 +554,6 @@ struct Raw<float> {
         link(lb, w);
     }
 };
-template <>
-struct Raw<__nv_bfloat16> {
-    uint4 pf[3], pb[3];
-    uint2 lf[3], lb[3];
-    __device__ __forceinline__ void load(const LpArgs& a, int mu, int64_t jf, int64_t jb, int64_t k) {
-        const uint4* in = (const uint4*)a.in;
-        const uint2* L = (const uint2*)a.links + (int64_t)mu * 3 * a.n;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) pf[c] = __ldg(in + c * a.n + jf);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) pb[c] = __ldg(in + c * a.n + jb);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) lf[c] = __ldg(L + c * a.n + k);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) lb[c] = __ldg(L + c * a.n + jb);
-    }
-    __device__ __forceinline__ static void spinor(const uint4 (&v)[3], float (&f)[24]) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            float2 t;
-            t = unpack_bf2(v[c].x); f[8 * c + 0] = t.x; f[8 * c + 1] = t.y;
-            t = unpack_bf2(v[c].y); f[8 * c + 2] = t.x; f[8 * c + 3] = t.y;
-            t = unpack_bf2(v[c].z); f[8 * c + 4] = t.x; f[8 * c + 5] = t.y;
-            t = unpack_bf2(v[c].w); f[8 * c + 6] = t.x; f[8 * c + 7] = t.y;
-        }
-    }
-    __device__ __forceinline__ static void link(const uint2 (&v)[3], float (&f)[12]) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            float2 t;
-            t = unpack_bf2(v[c].x); f[4 * c + 0] = t.x; f[4 * c + 1] = t.y;
-            t = unpack_bf2(v[c].y); f[4 * c + 2] = t.x; f[4 * c + 3] = t.y;
-        }
-    }
-    __device__ __forceinline__ void unpack(float (&f)[24], float (&b)[24], float (&u)[12], float (&w)[12]) const {
-        spinor(pf, f);
-        spinor(pb, b);
-        link(lf, u);
-        link(lb, w);
-    }
-};
-
 // the two hops of direction MU from raw operands (masked hops contribute 0)
 template <class S, int MU>
 __device__ __forceinline__ void raw_dir(const Raw<S>& r, bool hf, bool hb, float (&acc)[24]) {
@@ -688,6 +646,251 @@ __global__ void __launch_bounds__(128, MINB) k_dslash_lp_pipe(LpArgs a) {
                 e[0] = fmaf(tr, sv[2 * q], fmaf(ti, sv[2 * q + 1], e[0]));
                 e[1] = fmaf(tr, sv[2 * q + 1], fmaf(-ti, sv[2 * q], e[1]));
                 e[2] = fmaf(tr, tr, fmaf(ti, ti, e[2]));
+            }
+        }
+    }
+    if constexpr (EPI != EPI_NONE) {
+        float tot[3];
+        if (lp_reduce_last<3>(e, a.partial, a.counter, tot) && threadIdx.x == 0)
+            lp_finish<S, EPI>(a, a.st, tot);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Variant "two sites" (BF16 storage): a thread computes two sites, one in each
+// half of packed FP32 multiply-adds (fma.rn.f32x2, one issue slot for two).  BF16
+// is bound by instructions, not by HBM: one site per thread issues about 260 a hop
+// (144 of them arithmetic, 36 unpacking); packed, the arithmetic of two sites takes
+// 153, and BF16 unpacks into register pairs for free.  24^3 x 48 rest set 55.3 ->
+// 51.2 us (HBM floor 17.6), 32^3 x 64 whole lattice 164 -> 145: with three blocks of
+// 168 registers an SM (17 % of its warps) what is left waits for operands; keeping
+// the next direction's operands in registers was slower (61 us at two blocks).
+// ---------------------------------------------------------------------------
+struct p2 {            // one FP32 value of each of the two sites
+    unsigned long long v;
+};
+__device__ __forceinline__ p2 p2_make(float a, float b) {
+    p2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ p2 p2_all(float a) { return p2_make(a, a); }
+__device__ __forceinline__ void p2_get(p2 a, float& x, float& y) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.v));
+}
+__device__ __forceinline__ p2 p2_fma(p2 a, p2 b, p2 c) {
+    p2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ p2 operator*(p2 a, p2 b) {
+    p2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ p2 operator+(p2 a, p2 b) {
+    p2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ p2 operator-(p2 a, p2 b) { return p2_fma(b, p2_all(-1.f), a); }
+__device__ __forceinline__ p2 operator-(p2 a) { return a * p2_all(-1.f); }
+
+struct c2 {
+    p2 x, y;
+};
+
+// one direction's operands of the two sites, packed as loaded: words 0..11 of a
+// spinor are its complex numbers (re low, im high), words 0..5 of a link its rows 0, 1
+struct Raw2 {
+    uint32_t pf[2][12], pb[2][12], lf[2][6], lb[2][6];
+    __device__ __forceinline__ static void spinor(const LpArgs& a, int64_t j, bool on, uint32_t (&w)[12]) {
+        const uint4* in = (const uint4*)a.in;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const uint4 v = on ? __ldg(in + c * a.n + j) : make_uint4(0u, 0u, 0u, 0u);
+            w[4 * c] = v.x; w[4 * c + 1] = v.y; w[4 * c + 2] = v.z; w[4 * c + 3] = v.w;
+        }
+    }
+    __device__ __forceinline__ static void link(const uint2* L, int64_t n, int64_t j, uint32_t (&w)[6]) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const uint2 v = __ldg(L + c * n + j);
+            w[2 * c] = v.x; w[2 * c + 1] = v.y;
+        }
+    }
+    // a neighbour outside the set (-1) contributes zero
+    __device__ __forceinline__ void load(const LpArgs& a, int mu, const int2 (&nb)[2], const int64_t (&k)[2]) {
+        const uint2* L = (const uint2*)a.links + (int64_t)mu * 3 * a.n;
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            const bool hf = nb[m].x >= 0, hb = nb[m].y >= 0;
+            spinor(a, nb[m].x, hf, pf[m]);
+            spinor(a, nb[m].y, hb, pb[m]);
+            link(L, a.n, k[m], lf[m]);
+            link(L, a.n, hb ? (int64_t)nb[m].y : k[m], lb[m]);
+        }
+    }
+};
+
+__device__ __forceinline__ c2 bf2_word(uint32_t a, uint32_t b) {
+    return c2{p2_make(__uint_as_float(a << 16), __uint_as_float(b << 16)),
+              p2_make(__uint_as_float(a & 0xffff0000u), __uint_as_float(b & 0xffff0000u))};
+}
+
+// The three rows of -1/2 U: row 2 = -2 conj(row 0 x row 1).
+__device__ __forceinline__ void rebuild2(const uint32_t (&w)[2][6], c2 (&u)[3][3]) {
+    c2 A[3], N[3];     // -2 and +2 times row 0
+    p2 nb[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        u[0][c] = bf2_word(w[0][c], w[1][c]);
+        u[1][c] = bf2_word(w[0][3 + c], w[1][3 + c]);
+        A[c] = c2{u[0][c].x * p2_all(-2.f), u[0][c].y * p2_all(-2.f)};
+        N[c] = c2{u[0][c].x * p2_all(2.f), u[0][c].y * p2_all(2.f)};
+        nb[c] = -u[1][c].y;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const int i = (c + 1) % 3, j = (c + 2) % 3;
+        u[2][c].x = p2_fma(A[i].x, u[1][j].x, p2_fma(A[i].y, nb[j], p2_fma(N[j].x, u[1][i].x, A[j].y * u[1][i].y)));
+        u[2][c].y = p2_fma(N[i].x, u[1][j].y, p2_fma(N[i].y, u[1][j].x, p2_fma(A[j].x, u[1][i].y, A[j].y * u[1][i].x)));
+    }
+}
+
+// one hop of direction MU into the two sites' sums
+template <int MU, bool FWD>
+__device__ __forceinline__ void hop2(const uint32_t (&p)[2][12], const uint32_t (&l)[2][6], c2 (&acc)[12]) {
+    c2 h[2][3], u[3][3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const c2 s0 = bf2_word(p[0][c], p[1][c]), s1 = bf2_word(p[0][3 + c], p[1][3 + c]);
+        const c2 s2 = bf2_word(p[0][6 + c], p[1][6 + c]), s3 = bf2_word(p[0][9 + c], p[1][9 + c]);
+        auto add = [](c2 a, c2 b) { return c2{a.x + b.x, a.y + b.y}; };
+        auto sub = [](c2 a, c2 b) { return c2{a.x - b.x, a.y - b.y}; };
+        auto addi = [](c2 a, c2 b) { return c2{a.x - b.y, a.y + b.x}; };
+        auto subi = [](c2 a, c2 b) { return c2{a.x + b.y, a.y - b.x}; };
+        if (MU == 0) {
+            h[0][c] = FWD ? subi(s0, s3) : addi(s0, s3);
+            h[1][c] = FWD ? subi(s1, s2) : addi(s1, s2);
+        } else if (MU == 1) {
+            h[0][c] = FWD ? add(s0, s3) : sub(s0, s3);
+            h[1][c] = FWD ? sub(s1, s2) : add(s1, s2);
+        } else if (MU == 2) {
+            h[0][c] = FWD ? subi(s0, s2) : addi(s0, s2);
+            h[1][c] = FWD ? addi(s1, s3) : subi(s1, s3);
+        } else {
+            h[0][c] = FWD ? sub(s0, s2) : add(s0, s2);
+            h[1][c] = FWD ? sub(s1, s3) : add(s1, s3);
+        }
+    }
+    rebuild2(l, u);
+    c2 g[2][3];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        p2 neg[3];      // -h.y forward, -h.x backward
+#pragma unroll
+        for (int c = 0; c < 3; ++c) neg[c] = FWD ? -h[s][c].y : -h[s][c].x;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            c2 t;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const c2 w = FWD ? u[r][c] : u[c][r];
+                t.x = c == 0 ? w.x * h[s][c].x : p2_fma(w.x, h[s][c].x, t.x);
+                t.x = p2_fma(w.y, FWD ? neg[c] : h[s][c].y, t.x);
+                t.y = c == 0 ? w.x * h[s][c].y : p2_fma(w.x, h[s][c].y, t.y);
+                t.y = p2_fma(w.y, FWD ? h[s][c].x : neg[c], t.y);
+            }
+            g[s][r] = t;
+        }
+    }
+    // [g ; -+ X^dag g]
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const c2 a = g[0][c], b = g[1][c];
+        auto addto = [&](int k, c2 z) { acc[k] = c2{acc[k].x + z.x, acc[k].y + z.y}; };
+        auto subto = [&](int k, c2 z) { acc[k] = c2{acc[k].x - z.x, acc[k].y - z.y}; };
+        auto addi = [&](int k, c2 z) { acc[k] = c2{acc[k].x - z.y, acc[k].y + z.x}; };
+        auto subi = [&](int k, c2 z) { acc[k] = c2{acc[k].x + z.y, acc[k].y - z.x}; };
+        addto(c, a);
+        addto(3 + c, b);
+        if (MU == 0) {          // X^dag g = (-i g1, -i g0)
+            if (FWD) { addi(6 + c, b); addi(9 + c, a); } else { subi(6 + c, b); subi(9 + c, a); }
+        } else if (MU == 1) {   // (g1, -g0)
+            if (FWD) { subto(6 + c, b); addto(9 + c, a); } else { addto(6 + c, b); subto(9 + c, a); }
+        } else if (MU == 2) {   // (-i g0, i g1)
+            if (FWD) { addi(6 + c, a); subi(9 + c, b); } else { subi(6 + c, a); addi(9 + c, b); }
+        } else {
+            if (FWD) { subto(6 + c, a); subto(9 + c, b); } else { addto(6 + c, a); addto(9 + c, b); }
+        }
+    }
+}
+
+template <int MU>
+__device__ __forceinline__ void dir2(const LpArgs& a, const int2 (&nb)[2], const int64_t (&k)[2], c2 (&acc)[12]) {
+    Raw2 r;
+    r.load(a, MU, nb, k);
+    hop2<MU, true>(r.pf, r.lf, acc);
+    hop2<MU, false>(r.pb, r.lb, acc);
+}
+
+template <int EPI, int MINB>
+__global__ void __launch_bounds__(128, MINB) k_dslash_bf_two(LpArgs a) {
+    using S = __nv_bfloat16;
+    const bool skip = a.st != nullptr && a.st->done;
+    if (a.ran != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *a.ran = skip ? 0 : 1;
+    if (skip) return;
+    float e[3] = {0.f, 0.f, 0.f};
+    const int64_t span = 2 * (int64_t)blockDim.x;
+    for (int64_t base = blockIdx.x * span; base < a.n; base += (int64_t)gridDim.x * span) {
+        int64_t k[2] = {base + threadIdx.x, base + threadIdx.x + blockDim.x};
+        if (k[0] >= a.n) continue;
+        const bool two = k[1] < a.n;
+        if (!two) k[1] = k[0];
+        int4 n01[2], n23[2];
+#pragma unroll
+        for (int m = 0; m < 2; ++m) site_nbrs(a, k[m], n01[m], n23[m]);
+        c2 acc[12];
+#pragma unroll
+        for (int q = 0; q < 12; ++q) acc[q].x = acc[q].y = p2_all(0.f);
+        const int2 d0[2] = {make_int2(n01[0].x, n01[0].y), make_int2(n01[1].x, n01[1].y)};
+        const int2 d1[2] = {make_int2(n01[0].z, n01[0].w), make_int2(n01[1].z, n01[1].w)};
+        const int2 d2[2] = {make_int2(n23[0].x, n23[0].y), make_int2(n23[1].x, n23[1].y)};
+        const int2 d3[2] = {make_int2(n23[0].z, n23[0].w), make_int2(n23[1].z, n23[1].w)};
+        dir2<0>(a, d0, k, acc);
+        dir2<1>(a, d1, k, acc);
+        dir2<2>(a, d2, k, acc);
+        dir2<3>(a, d3, k, acc);
+        float out[2][24];
+#pragma unroll
+        for (int q = 0; q < 12; ++q) {
+            p2_get(acc[q].x, out[0][2 * q], out[1][2 * q]);
+            p2_get(acc[q].y, out[0][2 * q + 1], out[1][2 * q + 1]);
+        }
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            if (m == 1 && !two) break;
+            float self[24];
+            Store<S>::load_spinor(a.in, a.n, k[m], self);
+#pragma unroll
+            for (int q = 0; q < 24; ++q) out[m][q] = fmaf(a.diag, self[q], out[m][q]);
+            Store<S>::store_spinor(a.out, a.n, k[m], out[m]);
+            if (EPI != EPI_NONE) {
+                float w[24];
+                Store<S>::load_spinor(a.epi_vec, a.n, k[m], w);
+#pragma unroll
+                for (int q = 0; q < 12; ++q) {
+                    const float tr = out[m][2 * q], ti = out[m][2 * q + 1];
+                    if (EPI == EPI_DOT_RHAT_V) {
+                        e[0] = fmaf(w[2 * q], tr, fmaf(w[2 * q + 1], ti, e[0]));
+                        e[1] = fmaf(w[2 * q], ti, fmaf(-w[2 * q + 1], tr, e[1]));
+                    } else {
+                        e[0] = fmaf(tr, w[2 * q], fmaf(ti, w[2 * q + 1], e[0]));
+                        e[1] = fmaf(tr, w[2 * q + 1], fmaf(-ti, w[2 * q], e[1]));
+                        e[2] = fmaf(tr, tr, fmaf(ti, ti, e[2]));
+                    }
+                }
             }
         }
     }

@@ -19,6 +19,8 @@
 //   neighbours: int2 [n][mu] compact indices, -1 for a neighbour outside r.
 // One thread per site accumulates all eight hops in FP32 registers; the
 // kernel is HBM bound (384 B/site FP32, 192 B/site BF16 algorithmic).
+#include <type_traits>
+
 #include "lowp.cuh"
 
 namespace gs {
@@ -284,8 +286,9 @@ gs_status launch_lp_stencil(gs_ctx* c, LpArgs a, long long hops, int variant, lo
         }
     } else {
         // variants 1, 3, 4: thread per site with a register budget for
-        // 4, 6 or 8 blocks of 128 threads per SM; 5, 6: the same with the
-        // next direction's loads in flight (budget for 3 or 4 blocks)
+        // 4, 6 or 8 blocks of 128 threads per SM; 5, 6 (budget for 3 or 4
+        // blocks): FP32 the same with the next direction's loads in flight,
+        // BF16 two sites per thread
         const int b = lp_block(a.n, c->num_sms);
         int64_t g = (a.n + b - 1) / b;
         if (a.epi != EPI_NONE && g > kMaxRedBlocks) g = kMaxRedBlocks;
@@ -295,6 +298,13 @@ gs_status launch_lp_stencil(gs_ctx* c, LpArgs a, long long hops, int variant, lo
             case EPI_DOT_RHAT_V:                                                                 \
                 k_dslash_lp_site<S, EPI_DOT_RHAT_V, MB><<<(int)g, b, 0, c->stream>>>(a); break;  \
             default: k_dslash_lp_site<S, EPI_DOT_TS, MB><<<(int)g, b, 0, c->stream>>>(a); break; \
+        }
+#define GS_TWO_LAUNCH(MB)                                                                        \
+        switch (a.epi) {                                                                         \
+            case EPI_NONE: k_dslash_bf_two<EPI_NONE, MB><<<(int)g, b, 0, c->stream>>>(a); break; \
+            case EPI_DOT_RHAT_V:                                                                 \
+                k_dslash_bf_two<EPI_DOT_RHAT_V, MB><<<(int)g, b, 0, c->stream>>>(a); break;      \
+            default: k_dslash_bf_two<EPI_DOT_TS, MB><<<(int)g, b, 0, c->stream>>>(a); break;     \
         }
 #define GS_PIPE_LAUNCH(MB)                                                                       \
         switch (a.epi) {                                                                         \
@@ -307,15 +317,25 @@ gs_status launch_lp_stencil(gs_ctx* c, LpArgs a, long long hops, int variant, lo
             GS_SITE_LAUNCH(6)
         } else if (variant == 4) {
             GS_SITE_LAUNCH(8)
-        } else if (variant == 5) {
-            GS_PIPE_LAUNCH(3)
-        } else if (variant == 6) {
-            GS_PIPE_LAUNCH(4)
+        } else if (variant >= 5) {
+            if constexpr (std::is_same<S, __nv_bfloat16>::value) {
+                g = (g + 1) / 2;      // two sites per thread
+                if (variant == 5) {
+                    GS_TWO_LAUNCH(3)
+                } else {
+                    GS_TWO_LAUNCH(4)
+                }
+            } else if (variant == 5) {
+                GS_PIPE_LAUNCH(3)
+            } else {
+                GS_PIPE_LAUNCH(4)
+            }
         } else {
             GS_SITE_LAUNCH(4)
         }
 #undef GS_SITE_LAUNCH
 #undef GS_PIPE_LAUNCH
+#undef GS_TWO_LAUNCH
     }
     ++*launches;
     GS_CHECK_LAUNCH(c);
@@ -354,7 +374,8 @@ struct LpPlanData {
     long long hops = 0;    // in-set neighbour terms of one D application
     int variant = 0;       // stencil variant: 1/3/4 = thread per site (register budget for
                            // 4/6/8 blocks per SM), 2 = warp per direction, 5/6 = thread per
-                           // site with the next direction's loads in flight (3/4 blocks)
+                           // site with the next direction's loads in flight (FP32) or two
+                           // sites per thread (BF16), 3/4 blocks
     int2* nbr_r = nullptr;
     void* links = nullptr;
     LexDims lex{};         // the whole lattice: neighbours by arithmetic (identity plan)
