@@ -13,6 +13,7 @@
 //             K4 x += omega s, r = s - omega t, <rhat,r>, ||r||^2 -> beta, test,
 //             K5 p = r + beta (p - omega v).
 #include "gs_internal.cuh"
+#include "warp_sum.cuh"
 
 namespace gs {
 
@@ -21,30 +22,53 @@ namespace {
 constexpr int kBlas = 256;
 constexpr int kDotChunk = 8;   // vectors per block of the multi-dot
 
-// Block-reduce NV doubles; the last block gets the grand totals in thread 0.
+// A warp's sum of one double per thread of the block, and of n partials `ld`
+// apart (in block order).  Integer sums: a step of an FP64 shuffle tree takes
+// some 100 clocks, and every reduction here went through two trees and two
+// chains of 8 additions (k_norm2 over 12.6 MB, cold: 11.6 -> 10.0 us; the one-vector
+// k_multidot over 3 k entries: 9.4 -> 4.9 us).
+__device__ __forceinline__ double sum_of_block(const double* sm) {
+    const int lane = threadIdx.x & 31;
+    double x[kBlas / 32];
+#pragma unroll
+    for (int m = 0; m < kBlas / 32; ++m) x[m] = sm[m * 32 + lane];
+    return warp_sum<kBlas / 32>(x);
+}
+__device__ __forceinline__ double sum_of_partials(const double* part, int64_t ld, int n) {
+    const int lane = threadIdx.x & 31;
+    if (n <= 32) {
+        const double x[1] = {lane < n ? __ldcg(part + lane * ld) : 0.0};
+        return warp_sum<1>(x);
+    }
+    double t = 0.0;
+    for (int b0 = 0; b0 < n; b0 += 32 * 10) {
+        double x[10];
+#pragma unroll
+        for (int m = 0; m < 10; ++m) {
+            const int b = b0 + 32 * m + lane;
+            x[m] = b < n ? __ldcg(part + b * ld) : 0.0;
+        }
+        t += warp_sum<10>(x);
+    }
+    return t;
+}
+
+// Block-reduce NV <= 8 doubles; the last block gets the grand totals in thread 0.
 // Returns true (block-uniform) in the last block only.
 template <int NV>
 __device__ bool reduce_last(double (&v)[NV], RedScratch red, double (&tot)[NV]) {
-    __shared__ double sm[kBlas / 32][NV];
+    __shared__ double sm[NV][kBlas];
     __shared__ bool am_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nw = blockDim.x >> 5;
 #pragma unroll
-    for (int q = 0; q < NV; ++q) {
-        double x = v[q];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-        if (lane == 0) sm[warp][q] = x;
+    for (int q = 0; q < NV; ++q) sm[q][threadIdx.x] = v[q];
+    __syncthreads();
+    if (warp < NV) {
+        const double x = sum_of_block(sm[warp]);
+        if (lane == 0) red.partial[(int64_t)blockIdx.x * kMaxRedVals + warp] = x;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double* part = red.partial + (int64_t)blockIdx.x * kMaxRedVals;
-#pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            double x = 0.0;
-            for (int w = 0; w < nw; ++w) x += sm[w][q];
-            part[q] = x;
-        }
         __threadfence();
         const unsigned prev = atomicAdd(red.counter, 1u);
         am_last = (prev == gridDim.x - 1);
@@ -52,30 +76,14 @@ __device__ bool reduce_last(double (&v)[NV], RedScratch red, double (&tot)[NV]) 
     __syncthreads();
     if (!am_last) return false;
     __threadfence();
-    double s[NV];
-#pragma unroll
-    for (int q = 0; q < NV; ++q) s[q] = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
-        const volatile double* part = red.partial + (int64_t)b * kMaxRedVals;
-#pragma unroll
-        for (int q = 0; q < NV; ++q) s[q] += part[q];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-        double x = s[q];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-        if (lane == 0) sm[warp][q] = x;
+    if (warp < NV) {
+        const double x = sum_of_partials(red.partial + warp, kMaxRedVals, gridDim.x);
+        if (lane == 0) sm[warp][0] = x;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
 #pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            double x = 0.0;
-            for (int w = 0; w < nw; ++w) x += sm[w][q];
-            tot[q] = x;
-        }
+        for (int q = 0; q < NV; ++q) tot[q] = sm[q][0];
         *red.counter = 0u;
     }
     return true;
@@ -220,7 +228,7 @@ __global__ void k_multidot(const double2* __restrict__ X, int64_t ld, const doub
     // block (bx, c): the dots of vectors chunk c .. chunk c + chunk - 1 (chunk
     // <= 8) with y over the block's strided range (y read once for them); the
     // last block adds the per-block partials of every vector in block order
-    __shared__ double sm[kBlas / 32][2 * kDotChunk];
+    __shared__ double sm[2 * kDotChunk][kBlas];
     __shared__ bool am_last;
     const int k0 = blockIdx.y * chunk;
     const int nk = nvec - k0 < chunk ? nvec - k0 : chunk;
@@ -239,51 +247,29 @@ __global__ void k_multidot(const double2* __restrict__ X, int64_t ld, const doub
             }
         }
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int q = 0; q < 2 * kDotChunk; ++q) {
-        if (q < 2 * nk) {  // block-uniform
-            double v = a[q];
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-            if (lane == 0) sm[warp][q] = v;
-        }
+    for (int q = 0; q < 2 * kDotChunk; ++q)
+        if (q < 2 * nk) sm[q][threadIdx.x] = a[q];
+    __syncthreads();
+    for (int q = warp; q < 2 * nk; q += kBlas / 32) {
+        const double t = sum_of_block(sm[q]);
+        if (lane == 0) partial[(int64_t)(2 * k0 + q) * gridDim.x + blockIdx.x] = t;
     }
     __syncthreads();
-    const unsigned nblocks = gridDim.x * gridDim.y;
     if (threadIdx.x == 0) {
-        for (int q = 0; q < nk; ++q) {
-            double s0 = 0.0, s1 = 0.0;
-            for (int w = 0; w < nw; ++w) {
-                s0 += sm[w][2 * q];
-                s1 += sm[w][2 * q + 1];
-            }
-            double* part = partial + ((int64_t)(k0 + q) * gridDim.x + blockIdx.x) * 2;
-            part[0] = s0;
-            part[1] = s1;
-        }
         __threadfence();
         const unsigned prev = atomicAdd(counter, 1u);
-        am_last = (prev == nblocks - 1);
+        am_last = (prev == gridDim.x * gridDim.y - 1);
     }
     __syncthreads();
     if (!am_last) return;
     __threadfence();
-    for (int kk = threadIdx.x; kk < nvec; kk += blockDim.x) {
-        double s0 = 0.0, s1 = 0.0;
-        const double* part = partial + (int64_t)kk * gridDim.x * 2;
-        // L2 loads of the partials (all written before the counter reached
-        // nblocks); independent, so they are in flight together
-#pragma unroll 8
-        for (unsigned b = 0; b < gridDim.x; ++b) {
-            s0 += __ldcg(part + 2 * b);
-            s1 += __ldcg(part + 2 * b + 1);
-        }
-        if (accumulate) {
-            out[kk].x += s0;
-            out[kk].y += s1;
-        } else {
-            out[kk] = make_double2(s0, s1);
+    for (int q = warp; q < 2 * nvec; q += kBlas / 32) {
+        const double t = sum_of_partials(partial + (int64_t)q * gridDim.x, 1, gridDim.x);
+        if (lane == 0) {
+            double* o = (double*)out + q;
+            *o = accumulate ? *o + t : t;
         }
     }
     if (threadIdx.x == 0) *counter = 0u;

@@ -36,6 +36,7 @@
 #include <vector>
 
 #include "block12.cuh"
+#include "warp_sum.cuh"
 
 namespace gs {
 namespace {
@@ -59,31 +60,145 @@ struct BsrArgs {
     const double2* val;          // [nnzb][12][12], row-major blocks
 };
 
-constexpr int kBsrRows = 8;      // rows per block of 96 threads (12 per row)
+// What the rest solve's BiCGStab needs of v = A p (BSR_ALPHA: alpha = rho / <rhat, v>)
+// and t = A s (BSR_OMEGA: omega = <t, s> / <t, t>) beside the product.
+enum { BSR_NONE = 0, BSR_ALPHA = 1, BSR_OMEGA = 2 };
+struct BsrDots {
+    const double2* vec;          // rhat or s, in the output rows' order
+    BicgState* st;
+    RedScratch red;
+};
+
+constexpr int kBsrThreads = 128;
+constexpr int kBsrParts = 10;    // threads that share one component of a row
+constexpr int kBsrChunk = 32;    // stored blocks of a row taken at a time
 
 // out[k] = [addend[k]] + sign * sum_{b in row o0 + k, col j in the input
-// ranges} val_b in(j); thread (row, a) computes component a.
-__global__ void __launch_bounds__(96) k_bsr_apply(BsrArgs a) {
-    const int comp = threadIdx.x % 12;
-    const int rloc = threadIdx.x / 12;
-    for (int64_t k = (int64_t)blockIdx.x * kBsrRows + rloc; k < a.n_out;
-         k += (int64_t)gridDim.x * kBsrRows) {
+// ranges} val_b in(j).  One row per block: thread (a, p) takes products p,
+// p + 10, ... of component a, and the ten parts are added through shared memory.
+// The small levels are bound by latency and the FP64 pipe (a warp's instruction
+// holds a quarter of an SM for 80 clocks), so a row is spread over all four
+// quarters; with one thread per component, 8 rows a block, 240 rows of 7 blocks
+// kept 30 of 152 SMs busy on a chain of 168 multiply-adds a thread, 33.9 us.
+// The grid strides over the rows; large levels read 2304 bytes a block once.
+template <int DOTS>
+__global__ void __launch_bounds__(kBsrThreads) k_bsr_apply(BsrArgs a, BsrDots d) {
+    __shared__ double2 xs[kBsrChunk * 12];
+    __shared__ int32_t blk[kBsrChunk];
+    __shared__ double part[24][kBsrParts + 1];
+    __shared__ int count;
+    if (DOTS != BSR_NONE && d.st->done) return;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int comp = tid / kBsrParts, p0 = tid - comp * kBsrParts;
+    double e0 = 0.0, e1 = 0.0, e2 = 0.0;
+    for (int64_t k = blockIdx.x; k < a.n_out; k += gridDim.x) {
         const int64_t row = a.o0 + k;
         double2 acc = make_double2(0.0, 0.0);
-        const int32_t e = a.rowptr[row + 1];
-        for (int32_t b = a.rowptr[row]; b < e; ++b) {
-            const int64_t j = a.col[b];
-            const double2* src;
-            if (j >= a.a0 && j < a.a1) src = a.inA + (j - a.a0) * kSiteC;
-            else if (j >= a.a1 && j < a.b1) src = a.inB + (j - a.a1) * kSiteC;
-            else continue;
-            const double2* v = a.val + (int64_t)b * 144 + comp * 12;
+        const int32_t end = a.rowptr[row + 1];
+        for (int32_t b0 = a.rowptr[row]; b0 < end; b0 += kBsrChunk) {
+            if (tid < 32) {      // the chunk's blocks whose column is in a range, in order
+                const double2* src = nullptr;
+                if (b0 + lane < end) {
+                    const int64_t j = a.col[b0 + lane];
+                    if (j >= a.a0 && j < a.a1) src = a.inA + (j - a.a0) * kSiteC;
+                    else if (j >= a.a1 && j < a.b1) src = a.inB + (j - a.a1) * kSiteC;
+                }
+                const unsigned in = __ballot_sync(0xffffffffu, src != nullptr);
+                const int at = __popc(in & ((1u << lane) - 1u));
+                if (src) {
+                    blk[at] = b0 + lane;
 #pragma unroll
-            for (int q = 0; q < 12; ++q) cfma(acc, v[q], src[q]);
+                    for (int q = 0; q < 12; ++q) xs[at * 12 + q] = src[q];
+                }
+                if (lane == 0) count = __popc(in);
+            }
+            __syncthreads();
+            if (comp < 12) {
+                const int items = count * 12;
+#pragma unroll 9
+                for (int i = p0; i < items; i += kBsrParts) {
+                    const int m = i / 12;
+                    cfma(acc, a.val[(int64_t)blk[m] * 144 + comp * 12 + (i - m * 12)], xs[i]);
+                }
+            }
+            __syncthreads();
         }
-        if (a.negate) acc = make_double2(-acc.x, -acc.y);
-        if (a.addend) acc = cadd(acc, a.addend[k * kSiteC + comp]);
-        a.out[k * kSiteC + comp] = acc;
+        __syncthreads();         // the row before has been read, also past an empty row
+        if (comp < 12) {
+            part[2 * comp][p0] = acc.x;
+            part[2 * comp + 1][p0] = acc.y;
+        }
+        __syncthreads();
+        const int sum = tid / 5, g = tid - sum * 5;
+        if (sum < 24) part[sum][g] += part[sum][g + 5];
+        __syncthreads();
+        if (tid < 24) {          // real or imaginary part of one component each
+            double v = ((part[tid][0] + part[tid][1]) + (part[tid][2] + part[tid][3])) + part[tid][4];
+            if (a.negate) v = -v;
+            const int64_t at = k * 24 + tid;
+            if (a.addend) v += ((const double*)a.addend)[at];
+            ((double*)a.out)[at] = v;
+            if (DOTS != BSR_NONE) {
+                // <rhat, v> or <t, s>: this real number's share of the real and imaginary part
+                const double2 h = d.vec[k * 12 + tid / 2];
+                const bool im = tid & 1;
+                e0 = fma(im ? h.y : h.x, v, e0);
+                e1 = fma(im ? h.x : -h.y, v, e1);
+                if (DOTS == BSR_OMEGA) e2 = fma(v, v, e2);
+            }
+        }
+    }
+    if constexpr (DOTS != BSR_NONE) {
+        __shared__ bool am_last;
+        __shared__ double tot[3];
+        constexpr int NV = DOTS == BSR_OMEGA ? 3 : 2;
+        if (tid < 32) {
+            const double x0[1] = {e0}, x1[1] = {e1}, x2[1] = {e2};
+            const double t0 = warp_sum<1>(x0), t1 = warp_sum<1>(x1);
+            const double t2 = NV == 3 ? warp_sum<1>(x2) : 0.0;
+            if (lane == 0) {
+                double* q = d.red.partial + (int64_t)blockIdx.x * kMaxRedVals;
+                q[0] = t0;
+                q[1] = t1;
+                q[2] = t2;
+                __threadfence();
+                am_last = atomicAdd(d.red.counter, 1u) == gridDim.x - 1;
+            }
+        }
+        __syncthreads();
+        if (!am_last) return;
+        __threadfence();
+        const int q = tid >> 5;
+        if (q < NV) {            // one warp per value, partials in block order
+            double t = 0.0;
+            for (unsigned b0 = 0; b0 < gridDim.x; b0 += 32 * 8) {
+                double x[8];
+#pragma unroll
+                for (int m = 0; m < 8; ++m) {
+                    const unsigned b = b0 + 32 * m + lane;
+                    x[m] = b < gridDim.x ? __ldcg(d.red.partial + (int64_t)b * kMaxRedVals + q) : 0.0;
+                }
+                t += warp_sum<8>(x);
+            }
+            if (lane == 0) tot[q] = t;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            BicgState* st = d.st;
+            if (DOTS == BSR_ALPHA) {
+                st->alpha = cdiv(st->rho, make_double2(tot[0], tot[1]));
+                if (!isfinite(st->alpha.x) || !isfinite(st->alpha.y)) {
+                    st->status = GS_NONFINITE;
+                    st->done = 1;
+                    publish(st);
+                }
+            } else {
+                // t = A s, so <t, s> = conj(<s, t>): the sums above are <s, t>
+                st->omega = tot[2] > 0.0 ? make_double2(tot[0] / tot[2], -tot[1] / tot[2])
+                                         : make_double2(0.0, 0.0);
+            }
+            *d.red.counter = 0u;
+        }
     }
 }
 
@@ -369,8 +484,16 @@ int plain_blocks(gs_ctx* c, int64_t n, int block) { return grid_for(n, block, c-
 
 gs_status bsr_launch(gs_ctx* c, const BsrArgs& a) {
     if (a.n_out <= 0) return GS_OK;
-    const int g = grid_for(a.n_out, kBsrRows, c->num_sms * 32);
-    k_bsr_apply<<<g, 96, 0, c->stream>>>(a);
+    k_bsr_apply<BSR_NONE><<<grid_for(a.n_out, 1, c->num_sms * 32), kBsrThreads, 0, c->stream>>>(a, BsrDots{});
+    c->launches++;
+    GS_CHECK_LAUNCH(c);
+    return GS_OK;
+}
+
+// the product with its dot; one partial per block, so no more than kMaxRedBlocks
+template <int DOTS>
+gs_status bsr_launch_dots(gs_ctx* c, const BsrArgs& a, const BsrDots& d) {
+    k_bsr_apply<DOTS><<<grid_for(a.n_out, 1, kMaxRedBlocks), kBsrThreads, 0, c->stream>>>(a, d);
     c->launches++;
     GS_CHECK_LAUNCH(c);
     return GS_OK;
@@ -418,76 +541,67 @@ gs_status axpby(gs_ctx* c, cplx a, const double2* x, cplx b, double2* y, int64_t
 
 // z = A_rr^-1 b on a block-sparse level (levels >= 1): van der Vorst's
 // BiCGStab, x0 = 0, shadow residual b, stopped when ||s|| or ||r|| <=
-// tol ||b|| or after maxit steps (the last iterate is kept).
+// tol ||b|| or after maxit steps (the last iterate is kept).  Scalars stay on
+// the device and five launches make an iteration, queued two ahead of the
+// host's look at the `done` flag; scalars on the host took 5 dots with a copy
+// and a wait each, and 8 vector updates: 190 us an iteration on 240 sites.
 gs_status bsr_rest_bicgstab(gs_vcycle* vc, VLevel& L, const double2* b, double2* x) {
     gs_ctx* c = vc->c;
     const int64_t nb = L.nb, nr = L.n - L.nb, n = nr * kSiteC;
-    const size_t bytes = (size_t)n * sizeof(double2);
-    gs_status s;
-    GS_CUDA(c, cudaMemsetAsync(x, 0, bytes, c->stream));
-    double bnorm;
-    if ((s = vc_norm(vc, b, n, &bnorm)) != GS_OK) return s;
-    if (!isfinite(bnorm)) return set_err(c, GS_NONFINITE, "V-cycle: non-finite rest-set right-hand side");
-    vc->rest_solves++;
-    if (bnorm == 0.0) return GS_OK;
-    const double target = vc->rest_tol * bnorm;
-    GS_CUDA(c, cudaMemcpyAsync(L.r, b, bytes, cudaMemcpyDeviceToDevice, c->stream));
-    GS_CUDA(c, cudaMemcpyAsync(L.rhat, b, bytes, cudaMemcpyDeviceToDevice, c->stream));
-    GS_CUDA(c, cudaMemsetAsync(L.p, 0, bytes, c->stream));
-    GS_CUDA(c, cudaMemsetAsync(L.v, 0, bytes, c->stream));
+    gs_status s = ensure_inner(c, nr);
+    if (s != GS_OK) return s;
+    if (nr <= 0) {
+        vc->rest_solves++;
+        return GS_OK;
+    }
+    InnerWork w = c->inner;              // scalars, events and reduction scratch; the level's own vectors
+    w.r = L.r;
+    w.rhat = L.rhat;
+    w.p = L.p;
+    w.v = L.v;
+    w.s = L.s;
+    w.t = L.t;
     BsrArgs A = bsr_args(L);
     A.o0 = nb;
     A.n_out = nr;
     A.a0 = nb;
     A.a1 = L.n;
     A.b1 = L.n;
-    cplx rho_old = 1.0, alpha = 1.0, omega = 1.0;
-    int it = 0;
-    bool conv = false;
-    while (!conv && it < vc->rest_maxit) {
-        ++it;
-        cplx rho;
-        if ((s = vc_dot(vc, L.rhat, L.r, n, &rho)) != GS_OK) return s;
-        if (rho == 0.0) break;
-        const cplx beta = (rho / rho_old) * (alpha / omega);
-        // p = r + beta (p - omega v)
-        if ((s = axpby(c, -omega, L.v, 1.0, L.p, n)) != GS_OK) return s;
-        if ((s = axpby(c, 1.0, L.r, beta, L.p, n)) != GS_OK) return s;
-        A.out = L.v;
-        A.inA = L.p;
-        if ((s = bsr_launch(c, A)) != GS_OK) return s;
-        cplx rv;
-        if ((s = vc_dot(vc, L.rhat, L.v, n, &rv)) != GS_OK) return s;
-        alpha = rho / rv;
-        // s = r - alpha v
-        GS_CUDA(c, cudaMemcpyAsync(L.s, L.r, bytes, cudaMemcpyDeviceToDevice, c->stream));
-        if ((s = axpby(c, -alpha, L.v, 1.0, L.s, n)) != GS_OK) return s;
-        double sn;
-        if ((s = vc_norm(vc, L.s, n, &sn)) != GS_OK) return s;
-        if (!isfinite(sn)) return set_err(c, GS_NONFINITE, "V-cycle: non-finite rest-set residual");
-        if (sn <= target) {
-            if ((s = axpby(c, alpha, L.p, 1.0, x, n)) != GS_OK) return s;
-            conv = true;
-            break;
-        }
-        A.out = L.t;
-        A.inA = L.s;
-        if ((s = bsr_launch(c, A)) != GS_OK) return s;
-        cplx ts, tt;
-        if ((s = vc_dot(vc, L.t, L.s, n, &ts)) != GS_OK) return s;
-        if ((s = vc_dot(vc, L.t, L.t, n, &tt)) != GS_OK) return s;
-        omega = tt.real() > 0.0 ? ts / tt : cplx(0.0);
-        // x += alpha p + omega s ; r = s - omega t
-        if ((s = axpby(c, alpha, L.p, 1.0, x, n)) != GS_OK) return s;
-        if ((s = axpby(c, omega, L.s, 1.0, x, n)) != GS_OK) return s;
-        GS_CUDA(c, cudaMemcpyAsync(L.r, L.s, bytes, cudaMemcpyDeviceToDevice, c->stream));
-        if ((s = axpby(c, -omega, L.t, 1.0, L.r, n)) != GS_OK) return s;
-        rho_old = rho;
-        double rn;
-        if ((s = vc_norm(vc, L.r, n, &rn)) != GS_OK) return s;
-        if (!isfinite(rn)) return set_err(c, GS_NONFINITE, "V-cycle: non-finite rest-set residual");
-        conv = rn <= target;
-        if (omega == 0.0) break;
+    BsrArgs k1 = A, k3 = A;
+    k1.out = w.v;
+    k1.inA = w.p;
+    k3.out = w.t;
+    k3.inA = w.s;
+    const BsrDots d1 = {w.rhat, w.st, w.red}, d3 = {w.s, w.st, w.red};
+    volatile BicgPublic* pub = w.pub_host;
+    if ((s = launch_bicg_init(c, w, b, x, n, vc->rest_tol)) != GS_OK) return s;
+    GS_CUDA(c, cudaEventRecord(w.ev[3], c->stream));
+    constexpr int kDepth = 2;
+    int enq = 0;
+    while (enq < vc->rest_maxit) {
+        if (enq == 1) GS_CUDA(c, cudaEventSynchronize(w.ev[3]));   // init: b = 0 or not finite
+        if (enq >= kDepth) GS_CUDA(c, cudaEventSynchronize(w.ev[(enq - kDepth) % 3]));
+        if (enq >= 1 && pub->done) break;
+        if ((s = bsr_launch_dots<BSR_ALPHA>(c, k1, d1)) != GS_OK) return s;
+        if ((s = launch_bicg_s_update(c, w, x, n)) != GS_OK) return s;
+        if ((s = bsr_launch_dots<BSR_OMEGA>(c, k3, d3)) != GS_OK) return s;
+        if ((s = launch_bicg_xr_update(c, w, x, n)) != GS_OK) return s;
+        if ((s = launch_bicg_p_update(c, w, n)) != GS_OK) return s;
+        GS_CUDA(c, cudaEventRecord(w.ev[enq % 3], c->stream));
+        ++enq;
+    }
+    GS_CUDA(c, cudaEventSynchronize(enq > 0 ? w.ev[(enq - 1) % 3] : w.ev[3]));
+    if (!isfinite(pub->bb)) return set_err(c, GS_NONFINITE, "V-cycle: non-finite rest-set right-hand side");
+    vc->rest_solves++;
+    if (pub->bb == 0.0) return GS_OK;
+    if (pub->status == GS_NONFINITE) return set_err(c, GS_NONFINITE, "V-cycle: non-finite rest-set residual");
+    int it = pub->iter;
+    const bool conv = pub->done && pub->status == GS_OK;
+    if (pub->status == GS_BREAKDOWN && it < vc->rest_maxit) {
+        // rho = 0 is met at the start of the next iteration, omega = 0 at the end of its own
+        BicgState fin;
+        GS_CUDA(c, cudaMemcpy(&fin, w.st, sizeof fin, cudaMemcpyDeviceToHost));
+        if (fin.omega.x != 0.0 || fin.omega.y != 0.0) ++it;
     }
     vc->rest_iters += it;
     if (it > vc->rest_max_seen) vc->rest_max_seen = it;
