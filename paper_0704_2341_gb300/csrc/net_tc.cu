@@ -16,18 +16,26 @@
 // (leading byte offset), 8-row groups 768 bytes apart (stride byte offset).
 // The input activations are BF16 ([V][96][3] complex as bf16x2).
 //
-// Warp roles.  Warps 0-14 gather and transport: at chunk j they gather the
-// raw neighbour rows of chunk j + 2 by cp.async (three raw buffers; the links
-// of a transport once, two link buffers by transport parity), transport
-// chunk j into the A stage (two stages, reused once the tensor core has
-// committed the chunk two back) and arrive on the stage's full barrier; one
-// named barrier per chunk among these warps orders the raw buffers.  Warp 15
-// moves B_j by a bulk copy and issues the chunk's six MMAs as soon as the
-// stage is full, then commits them to the stage's done barrier, so the MMAs
-// never wait for a block barrier.  Every wait is bounded (the context's wait
+// Warp roles.  A tile is 85 sites (255 of the 256 GEMM rows) in 11 groups of
+// 8; warps 0-10 own a group each, so a warp depends on no other until the
+// tensor core: at chunk j it gathers its sites' raw rows of chunk j + 3 by
+// cp.async (four raw buffers), transports chunk j into the A stage (two
+// stages, reused once the tensor core has committed the chunk two back) and
+// arrives on the stage's full barrier.  Warp 11 moves B_j by a bulk copy and
+// issues the chunk's six MMAs as soon as the stage is full, then commits them
+// to the stage's done barrier.  Every wait is bounded (the context's wait
 // limit, GS_OPT_WAIT_LIMIT_US, 1 s by default); on a timeout the kernel
 // stops, waits (bounded) for the MMAs it committed, frees its tensor memory
 // and raises err.
+//
+// Bound by the transport's instructions: 36 multiply-adds a row and hop,
+// against 7.3 % of the time in the tensor core at its peak.  With the rows of
+// a site spread over 15 warps a (row, site) item took 172 warp instructions
+// (index arithmetic, links reloaded, gather loop) and a block barrier a chunk
+// left the schedulers idle half the time.  Here a lane keeps its site's link in
+// registers for a transport's four chunks, each component twice, and two rows
+// share every multiply-add (fma.rn.f32x2).  16^3 x 32 under the profiler: 1.11 ms
+// -> TC_AFTER ms.
 #include <cuda_bf16.h>
 #include <stdint.h>
 
@@ -37,12 +45,17 @@ namespace gs {
 namespace {
 
 constexpr int kRows = 256;                       // GEMM rows per tile
+constexpr int kTileSites = 85;                   // sites per tile (row 255 is not used)
 constexpr int kRC = 96;                          // 4 C, C = 24
 constexpr int kN = 192;                          // real output columns
 constexpr int kQ = 24;                           // input rows per chunk
 constexpr int kKC = 2 * kQ;                      // real K per chunk
 constexpr int kChunks = 36;                      // 9 transports x 4 quarters
-constexpr int kSites = 88;                       // site slots of a tile (at most 86 used)
+constexpr int kStageWarps = 11;                  // gather + transport, 8 sites each; warp 11 issues B and the MMAs
+constexpr int kThreads = 32 * (kStageWarps + 1);
+constexpr int kSites = 8 * kStageWarps;          // site slots of a tile
+constexpr int kRaw = 4;                          // raw buffers
+constexpr int kPieces = 8 * 18;                  // 16-byte pieces of a warp's raw rows of a chunk
 constexpr uint32_t kSBO = (kKC / 8) * 128;       // 768
 constexpr uint32_t kABytes = kRows * kKC * 2;    // 24576
 constexpr uint32_t kBBytes = kN * kKC * 2;       // 18432
@@ -50,14 +63,11 @@ constexpr uint32_t kPStride = kQ * 3 * 4 + 16;   // 304: raw rows of one site (+
 constexpr uint32_t kPBytes = kSites * kPStride;  // 26752
 constexpr uint32_t kUBytes = kSites * 9 * 8;     // 6336
 // dynamic shared memory map (offsets from a 128-byte aligned base): A and B
-// stages x 2, raw rows x 3, links x 2, neighbour table
-constexpr uint32_t kOffA = 0, kOffB = 2 * kABytes, kOffP = kOffB + 2 * kBBytes, kOffU = kOffP + 3 * kPBytes,
+// stages x 2, raw rows x 4, links x 2, neighbour table
+constexpr uint32_t kOffA = 0, kOffB = 2 * kABytes, kOffP = kOffB + 2 * kBBytes, kOffU = kOffP + kRaw * kPBytes,
                    kOffY = kOffU + 2 * kUBytes, kSmemUsed = kOffY + 9 * kSites * 4;
 constexpr size_t kSmem = kSmemUsed + 128;
-constexpr int kThreads = 512;
-constexpr int kStageWarps = 15;                  // gather + transport; warp 15 issues B and the MMAs
-constexpr int kStageThreads = kStageWarps * 32;
-constexpr int kHalfItems = 11 * 3 * 2;           // (8 site slots) x (8 rows) x (first / second row of a lane)
+static_assert(3 * kTileSites <= kRows && kTileSites <= kSites, "rows of a tile");
 static_assert(kSmem <= 227 * 1024, "shared memory");
 
 __device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -112,123 +122,120 @@ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {  // conj(a) b
     return make_float2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
 }
 
-// raw rows of chunk j of the tile into raw buffer j % 3, and with the first
-// quarter of a transport its links into link buffer (transport & 1); issued
-// by the transport warps, one commit group per chunk
-__device__ __forceinline__ void gather(unsigned char* base, int j, const __nv_bfloat162* __restrict__ in,
-                                       const float2* __restrict__ U32, int64_t xs0, int nsite) {
-    const int d = j >> 2, qt = j & 3;
-    const int* Y = (const int*)(base + kOffY) + d * kSites;
-    const uint32_t P = su32(base + kOffP + (j % 3) * kPBytes);
-    for (int i = threadIdx.x; i < nsite * 18; i += kStageThreads) {
-        const int sl = i / 18, pc = i - sl * 18;
-        const unsigned char* src = (const unsigned char*)(in + ((int64_t)Y[sl] * kRC + kQ * qt) * 3) + pc * 16;
-        cp_async16(P + sl * kPStride + pc * 16, src);
-    }
-    if (d > 0 && qt == 0) {  // links of transport d, kept for its four quarters
-        const int mu = (d - 1) & 3;
-        const uint32_t Ub = su32(base + kOffU + (d & 1) * kUBytes);
-        for (int i = threadIdx.x; i < nsite * 9; i += kStageThreads) {
-            const int sl = i / 9, e = i - sl * 9;
-            const int64_t ls = d <= 4 ? xs0 + sl : (int64_t)Y[sl];
-            cp_async8(Ub + (sl * 9 + e) * 8, U32 + (ls * 4 + mu) * 9 + e);
+// The raw rows of chunk j of warp `sg`'s sites into raw buffer j % kRaw, and with
+// the first quarter of a transport its links into link buffer (transport & 1);
+// one commit group per chunk (an empty one past the last).
+__device__ __forceinline__ void gather(unsigned char* base, int sg, int lane, int j,
+                                       const __nv_bfloat162* __restrict__ in, const float2* __restrict__ U32,
+                                       int64_t xs0, int nsite) {
+    if (j < kChunks) {
+        const int d = j >> 2, qt = j & 3;
+        const int* Y = (const int*)(base + kOffY) + d * kSites;
+        const uint32_t P = su32(base + kOffP + (j % kRaw) * kPBytes);
+#pragma unroll
+        for (int t = 0; t < (kPieces + 31) / 32; ++t) {
+            const int i = lane + 32 * t;
+            const int sl = 8 * sg + i / 18, pc = i % 18;
+            if (i < kPieces && sl < nsite)
+                cp_async16(P + sl * kPStride + pc * 16,
+                           (const unsigned char*)(in + ((int64_t)Y[sl] * kRC + kQ * qt) * 3) + pc * 16);
+        }
+        if (d > 0 && qt == 0) {
+            const int mu = (d - 1) & 3;
+            const uint32_t Ub = su32(base + kOffU + (d & 1) * kUBytes);
+            for (int i = lane; i < 72; i += 32) {
+                const int sl = 8 * sg + i / 9, e = i % 9;
+                if (sl < nsite) {
+                    const int64_t ls = d <= 4 ? xs0 + sl : (int64_t)Y[sl];
+                    cp_async8(Ub + (sl * 9 + e) * 8, U32 + (ls * 4 + mu) * 9 + e);
+                }
+            }
         }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// Transport one chunk (24 input rows) of the raw rows in shared memory into
-// the A stage.  MODE 0: identity, 1: U_mu(x) p (forward hop), 2: U^dag p
-// (backward hop; the link is the neighbour's).  Half-items = (8 site slots)
-// x (8 input rows) x (first or second row of a lane): lane = (site j, row q)
-// handles row q or q + 4 of its site; the 66 half-items go in contiguous runs
-// of four or five to the 15 transport warps, so a warp loads a site's link at
-// most twice.  The bf16x2 stores of a warp land in 32 distinct banks (bank =
-// 4 (row mod 8) + q).  Each output colour is one FMA chain per real
-// component; the row bounds are checked only on the tile's edge items.
-__device__ __forceinline__ uint32_t core_row(int r) { return (uint32_t)((r >> 3) * kSBO + (r & 7) * 16); }
-
-// t = sum_c m_c p_c  (m_c = U[a][c]: forward) or sum_c conj(m_c) p_c (backward)
-template <bool CONJ>
-__device__ __forceinline__ float2 row3(float2 m0, float2 m1, float2 m2, float2 p0, float2 p1, float2 p2) {
-    const float s = CONJ ? -1.f : 1.f;
-    float re = m0.x * p0.x;
-    re = fmaf(-s * m0.y, p0.y, re);
-    re = fmaf(m1.x, p1.x, re);
-    re = fmaf(-s * m1.y, p1.y, re);
-    re = fmaf(m2.x, p2.x, re);
-    re = fmaf(-s * m2.y, p2.y, re);
-    float im = m0.x * p0.y;
-    im = fmaf(s * m0.y, p0.x, im);
-    im = fmaf(m1.x, p1.y, im);
-    im = fmaf(s * m1.y, p1.x, im);
-    im = fmaf(m2.x, p2.y, im);
-    im = fmaf(s * m2.y, p2.x, im);
-    return make_float2(re, im);
+// two floats for the packed multiply-add
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ void fma2(uint64_t& r, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(r) : "l"(a), "l"(b));
 }
 
-template <int MODE>
-__device__ __forceinline__ void stage_chunk(const unsigned char* P, const float2* Ub, unsigned char* a_s, int warp,
-                                            int sj, int kq, int off, int nsite) {
-    const int h0 = warp * kHalfItems / kStageWarps, h1 = (warp + 1) * kHalfItems / kStageWarps;
-    int cached = -1;
-    float2 u[9];
-    for (int hi = h0; hi < h1; ++hi) {
-        const int sg = hi / 6, rem = hi - 6 * sg, kg = rem >> 1, h2 = rem & 1;
-        const int sl = 8 * sg + sj;
-        const int r0 = 3 * sl - off;
-        if (r0 >= kRows) continue;
-        const bool have = sl < nsite;
-        if (MODE != 0 && have && sg != cached) {
+// A lane's transport matrix, U (forward hop) or U^dag (backward hop), every
+// component in both halves of a register pair.
+struct Link2 {
+    uint64_t x[9], y[9], ny[9];
+};
+__device__ __forceinline__ void load_link2(Link2& m, const float2* u, bool dagger) {
 #pragma unroll
-            for (int e = 0; e < 9; ++e) u[e] = Ub[sl * 9 + e];
-            cached = sg;
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float2 v = u[dagger ? 3 * c + a : 3 * a + c];
+            const float im = dagger ? -v.y : v.y;
+            m.x[3 * a + c] = pack2(v.x, v.x);
+            m.y[3 * a + c] = pack2(im, im);
+            m.ny[3 * a + c] = pack2(-im, -im);
         }
-        const int kk = 8 * kg + 4 * h2 + kq;
-        // core matrix column of k' = 2 kk: (2 kk / 8) * 128 + (2 kk % 8) * 2
-        const uint32_t ok = (uint32_t)((2 * kg + h2) * 128 + 4 * kq);
-        float2 t0 = make_float2(0.f, 0.f), t1 = t0, t2 = t0;
-        if (have) {
-            const __nv_bfloat162* pr = (const __nv_bfloat162*)(P + sl * kPStride) + kk * 3;
-            const float2 p0 = __bfloat1622float2(pr[0]), p1 = __bfloat1622float2(pr[1]),
-                         p2 = __bfloat1622float2(pr[2]);
-            if (MODE == 0) {
-                t0 = p0;
-                t1 = p1;
-                t2 = p2;
-            } else if (MODE == 1) {
-                t0 = row3<false>(u[0], u[1], u[2], p0, p1, p2);
-                t1 = row3<false>(u[3], u[4], u[5], p0, p1, p2);
-                t2 = row3<false>(u[6], u[7], u[8], p0, p1, p2);
-            } else {
-                t0 = row3<true>(u[0], u[3], u[6], p0, p1, p2);
-                t1 = row3<true>(u[1], u[4], u[7], p0, p1, p2);
-                t2 = row3<true>(u[2], u[5], u[8], p0, p1, p2);
-            }
-        }
-        if (r0 >= 0 && r0 + 2 < kRows) {
-            *(__nv_bfloat162*)(a_s + core_row(r0) + ok) = __floats2bfloat162_rn(t0.x, t0.y);
-            *(__nv_bfloat162*)(a_s + core_row(r0 + 1) + ok) = __floats2bfloat162_rn(t1.x, t1.y);
-            *(__nv_bfloat162*)(a_s + core_row(r0 + 2) + ok) = __floats2bfloat162_rn(t2.x, t2.y);
-        } else {
-            if (r0 >= 0) *(__nv_bfloat162*)(a_s + core_row(r0) + ok) = __floats2bfloat162_rn(t0.x, t0.y);
-            if (r0 + 1 >= 0 && r0 + 1 < kRows)
-                *(__nv_bfloat162*)(a_s + core_row(r0 + 1) + ok) = __floats2bfloat162_rn(t1.x, t1.y);
-            if (r0 + 2 < kRows) *(__nv_bfloat162*)(a_s + core_row(r0 + 2) + ok) = __floats2bfloat162_rn(t2.x, t2.y);
-        }
+}
+
+// Transport one chunk (24 input rows) of a lane's site: rows kq, kq + 4, ...;
+// lane = (site j, kq).  A's rows are 3 site + colour; the bf16x2 stores of a warp
+// land in 32 distinct banks (bank = 4 (row mod 8) + kq).
+__device__ __forceinline__ uint32_t core_row(int r) { return (uint32_t)((r >> 3) * kSBO + (r & 7) * 16); }
+
+__device__ __forceinline__ void stage_copy(const uint32_t* raw, unsigned char* a_s, int r0, int kq) {
+#pragma unroll
+    for (int h = 0; h < 6; ++h) {
+        const uint32_t ok = (uint32_t)(h * 128 + 4 * kq);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) *(uint32_t*)(a_s + core_row(r0 + c) + ok) = raw[(4 * h + kq) * 3 + c];
     }
 }
 
-// named barrier of the transport warps with an OR of v over them
-__device__ __forceinline__ bool stage_sync_or(int v) {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\tbar.red.or.pred q, 1, %2, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(r)
-        : "r"(v), "n"(kStageThreads)
-        : "memory");
-    return r != 0;
+__device__ __forceinline__ void stage_transport(const uint32_t* raw, const Link2& m, unsigned char* a_s, int r0,
+                                                int kq) {
+#pragma unroll
+    for (int g = 0; g < 3; ++g) {
+        uint64_t px[3], py[3];     // rows 8 g + kq and 8 g + 4 + kq
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const uint32_t w0 = raw[(8 * g + kq) * 3 + c], w1 = raw[(8 * g + 4 + kq) * 3 + c];
+            px[c] = pack2(__uint_as_float(w0 << 16), __uint_as_float(w1 << 16));
+            py[c] = pack2(__uint_as_float(w0 & 0xffff0000u), __uint_as_float(w1 & 0xffff0000u));
+        }
+        const uint32_t ok = (uint32_t)(2 * g * 128 + 4 * kq);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            uint64_t re = mul2(m.x[3 * a], px[0]), im = mul2(m.x[3 * a], py[0]);
+            fma2(re, m.ny[3 * a], py[0]);
+            fma2(im, m.y[3 * a], px[0]);
+#pragma unroll
+            for (int c = 1; c < 3; ++c) {
+                fma2(re, m.x[3 * a + c], px[c]);
+                fma2(im, m.x[3 * a + c], py[c]);
+                fma2(re, m.ny[3 * a + c], py[c]);
+                fma2(im, m.y[3 * a + c], px[c]);
+            }
+            const float2 r = unpack2(re), i = unpack2(im);
+            *(__nv_bfloat162*)(a_s + core_row(r0 + a) + ok) = __floats2bfloat162_rn(r.x, i.x);
+            *(__nv_bfloat162*)(a_s + core_row(r0 + a) + ok + 128) = __floats2bfloat162_rn(r.y, i.y);
+        }
+    }
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -241,7 +248,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // s; mdone: the MMAs of the stage's chunk completed (tcgen05.commit)
     __shared__ __align__(8) uint64_t afull[2], bfull[2], mdone[2];
     __shared__ uint32_t tslot;
-    __shared__ uint32_t committed;   // chunks whose MMAs warp 15 has committed
+    __shared__ uint32_t committed;   // chunks whose MMAs warp 11 has committed
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
         for (int s = 0; s < 2; ++s) {
@@ -261,18 +268,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tslot;
 
-    const int64_t rows = 3 * V;
-    const int64_t ntiles = (rows + kRows - 1) / kRows;
+    const int64_t ntiles = (V + kTileSites - 1) / kTileSites;
     uint32_t g = 0;  // chunks of the tiles before this one (stage = g & 1, use = g >> 1)
     int bad = 0;
     const int kq = lane & 3, sj = lane >> 2;
     for (int64_t tile = blockIdx.x; tile < ntiles && !bad; tile += gridDim.x) {
-        const int64_t row0 = tile * kRows;
-        const int64_t xs0 = row0 / 3;
-        const int off = (int)(row0 - 3 * xs0);
-        int64_t xl = (row0 + kRows - 1) / 3;
-        if (xl > V - 1) xl = V - 1;
-        const int nsite = (int)(xl - xs0 + 1);
+        const int64_t xs0 = tile * kTileSites;
+        const int nsite = (int)(V - xs0 < kTileSites ? V - xs0 : kTileSites);
         // neighbour site of every (transport, site) of the tile
         int* Y = (int*)(base + kOffY);
         for (int i = tid; i < 9 * kSites; i += kThreads) {
@@ -284,35 +286,41 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         __syncthreads();
         if (warp < kStageWarps) {
-            gather(base, 0, in, U32, xs0, nsite);
-            gather(base, 1, in, U32, xs0, nsite);
+            for (int j = 0; j < kRaw - 1; ++j) gather(base, warp, lane, j, in, U32, xs0, nsite);
+            const int sl = 8 * warp + sj;
+            Link2 m;
             for (int j = 0; j < kChunks; ++j) {
                 const uint32_t gj = g + (uint32_t)j, s = gj & 1u, u = gj >> 1;
-                if (j + 1 < kChunks) asm volatile("cp.async.wait_group 1;" ::: "memory");
-                else asm volatile("cp.async.wait_group 0;" ::: "memory");
-                // the MMAs of chunk gj - 2 read this A stage: one thread waits
-                // for their commit, the named barrier passes the news on (and
-                // that every transport warp is done with chunk j - 1's raw rows)
-                if (tid == 0 && gj >= 2 && !mbar_wait(su32(&mdone[s]), (u - 1) & 1u, wait_ns)) bad = 1;
-                if (stage_sync_or(bad)) {
+                // chunk j's raw rows are in, and the warp is done with chunk j - 1's,
+                // whose buffer chunk j + 3 takes
+                asm volatile("cp.async.wait_group %0;" ::"n"(kRaw - 2) : "memory");
+                __syncwarp();
+                gather(base, warp, lane, j + kRaw - 1, in, U32, xs0, nsite);
+                // the MMAs of chunk gj - 2 read this A stage
+                if (gj >= 2 && !mbar_wait(su32(&mdone[s]), (u - 1) & 1u, wait_ns)) bad = 1;
+                if (__any_sync(0xffffffffu, bad)) {
                     bad = 1;
                     break;
                 }
-                if (j + 2 < kChunks) gather(base, j + 2, in, U32, xs0, nsite);
                 const int d = j >> 2;
-                const unsigned char* P = base + kOffP + (j % 3) * kPBytes;
-                const float2* Ub = (const float2*)(base + kOffU + (d & 1) * kUBytes);
+                const uint32_t* raw = (const uint32_t*)(base + kOffP + (j % kRaw) * kPBytes + sl * kPStride);
                 unsigned char* a_s = base + kOffA + s * kABytes;
-                if (d == 0) stage_chunk<0>(P, Ub, a_s, warp, sj, kq, off, nsite);
-                else if (d <= 4) stage_chunk<1>(P, Ub, a_s, warp, sj, kq, off, nsite);
-                else stage_chunk<2>(P, Ub, a_s, warp, sj, kq, off, nsite);
+                if (sl < nsite) {
+                    if (d == 0) {
+                        stage_copy(raw, a_s, 3 * sl, kq);
+                    } else {
+                        if ((j & 3) == 0)
+                            load_link2(m, (const float2*)(base + kOffU + (d & 1) * kUBytes) + sl * 9, d > 4);
+                        stage_transport(raw, m, a_s, 3 * sl, kq);
+                    }
+                }
                 // the tensor core reads the stage through the async proxy
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(&afull[s])) : "memory");
             }
         } else if (lane == 0) {
-            // warp 15: B_j by bulk copy, then the chunk's MMAs once A and B are in
+            // warp 11: B_j by bulk copy, then the chunk's MMAs once A and B are in
             for (int j = 0; j < kChunks; ++j) {
                 const uint32_t gj = g + (uint32_t)j, s = gj & 1u, u = gj >> 1;
                 if (gj >= 2 && !mbar_wait(su32(&mdone[s]), (u - 1) & 1u, wait_ns)) {  // B stage s free
@@ -364,13 +372,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (__syncthreads_or(bad)) bad = 1;
         asm volatile("tcgen05.fence::after_thread_sync;");
         if (!bad) {
-            // warp w reads lanes 32 (w % 4) .. + 31 of accumulator (w / 4) % 2, columns half w / 8
-            const int q = (warp >> 2) & 1, wq = warp & 3, ch = warp >> 3;
-            const int r = 128 * q + 32 * wq + lane;
-            const int64_t p = row0 + r;
-            const int64_t x = p / 3;
-            const int a = (int)(p - 3 * x);
-            for (int c = ch * (kN / 2); c < (ch + 1) * (kN / 2); c += 32) {
+            // warp w reads lanes 32 (w % 4) .. + 31; the 12 (accumulator, 32 columns)
+            // pieces of those lanes go to its three warps
+            const int wq = warp & 3;
+            for (int u = warp >> 2; u < 2 * kN / 32; u += 3) {
+                const int q = u / (kN / 32), c = 32 * (u - q * (kN / 32));
+                const int r = 128 * q + 32 * wq + lane;
                 uint32_t v[32];
                 asm volatile(
                     "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
@@ -382,8 +389,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                       "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
                     : "r"(tmem + ((uint32_t)(32 * wq) << 16) + (uint32_t)(q * kN + c)));
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (p < rows) {
-                    float2* dst = out + (x * kRC + c / 2) * 3 + a;
+                if (r < 3 * nsite) {
+                    float2* dst = out + ((xs0 + r / 3) * kRC + c / 2) * 3 + r % 3;
 #pragma unroll
                     for (int i = 0; i < 16; ++i)
                         dst[3 * i] = make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
@@ -891,7 +898,7 @@ gs_status net_phi_tc(gs_ctx* c, const float2* in, float2* phi, const __nv_bfloat
 gs_status net_conv_tc(gs_ctx* c, const __nv_bfloat162* in, float2* out, const __nv_bfloat16* Bw, const float2* U32,
                       const int2* nbr, int64_t V, int* err) {
     GS_CUDA(c, cudaFuncSetAttribute(k_net_conv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem));
-    const int64_t ntiles = (3 * V + kRows - 1) / kRows;
+    const int64_t ntiles = (V + kTileSites - 1) / kTileSites;
     const int grid = (int)(ntiles < c->num_sms ? ntiles : c->num_sms);
     k_net_conv_tc<<<grid, kThreads, kSmem, c->stream>>>(in, out, Bw, U32, nbr, V, err, c->wait_ns);
     c->launches++;
