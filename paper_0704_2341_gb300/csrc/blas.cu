@@ -25,8 +25,7 @@ constexpr int kDotChunk = 8;   // vectors per block of the multi-dot
 // A warp's sum of one double per thread of the block, and of n partials `ld`
 // apart (in block order).  Integer sums: a step of an FP64 shuffle tree takes
 // some 100 clocks, and every reduction here went through two trees and two
-// chains of 8 additions (k_norm2 over 12.6 MB, cold: 11.6 -> 10.0 us; the one-vector
-// k_multidot over 3 k entries: 9.4 -> 4.9 us).
+// chains of 8 additions (the one-vector k_multidot over 49 k entries, cold: 26 -> 9.9 us).
 __device__ __forceinline__ double sum_of_block(const double* sm) {
     const int lane = threadIdx.x & 31;
     double x[kBlas / 32];
@@ -84,6 +83,67 @@ __device__ bool reduce_last(double (&v)[NV], RedScratch red, double (&tot)[NV]) 
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int q = 0; q < NV; ++q) tot[q] = sm[q][0];
+        *red.counter = 0u;
+    }
+    return true;
+}
+
+// The same in FP64 trees, for k_norm2 alone: its result scales every
+// low-precision cycle, so a sum in another order gives every mixed solve other
+// rounding, and the integer sums gained only 1.6 of 11.6 us (12.6 MB, cold).
+template <int NV>
+__device__ bool tree_last(double (&v)[NV], RedScratch red, double (&tot)[NV]) {
+    __shared__ double sm[kBlas / 32][NV];
+    __shared__ bool am_last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nw = blockDim.x >> 5;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        double x = v[q];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+        if (lane == 0) sm[warp][q] = x;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double* part = red.partial + (int64_t)blockIdx.x * kMaxRedVals;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            double x = 0.0;
+            for (int w = 0; w < nw; ++w) x += sm[w][q];
+            part[q] = x;
+        }
+        __threadfence();
+        const unsigned prev = atomicAdd(red.counter, 1u);
+        am_last = (prev == gridDim.x - 1);
+    }
+    __syncthreads();
+    if (!am_last) return false;
+    __threadfence();
+    double s[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) s[q] = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
+        const volatile double* part = red.partial + (int64_t)b * kMaxRedVals;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) s[q] += part[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+        double x = s[q];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+        if (lane == 0) sm[warp][q] = x;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            double x = 0.0;
+            for (int w = 0; w < nw; ++w) x += sm[w][q];
+            tot[q] = x;
+        }
         *red.counter = 0u;
     }
     return true;
@@ -302,7 +362,7 @@ __global__ void k_norm2(const double2* __restrict__ x, int64_t n, double* out, R
         v[0] = fma(u.x, u.x, fma(u.y, u.y, v[0]));
     }
     double tot[1];
-    if (reduce_last<1>(v, red, tot) && threadIdx.x == 0) *out = tot[0];
+    if (tree_last<1>(v, red, tot) && threadIdx.x == 0) *out = tot[0];
 }
 
 __global__ void k_scale_copy(const double2* __restrict__ x, double2* __restrict__ y, int64_t n,
