@@ -60,8 +60,8 @@ PERM_NAMES = ["P_I", "P_II", "P_I^T", "P_II^T"]
 # DRAM traffic per launch from one ncu capture, per profiled kernel family
 # (3: the persistent FP64 BiCGStab, the step's dominant kernel), with the hash
 # of the sources it was taken on; other families report no traffic
-NCU_SUMMARY = {3: (os.path.join(ROOT, "profiles", "bicg_persistent_f64_8x4_traffic.txt"),
-                   ("persistent.cu", "dslash_f64.cuh", "gridsync.cuh"))}
+NCU_SUMMARY = {3: (os.path.join(ROOT, "profiles", "bicg_persistent_fx_8x4_traffic.txt"),
+                   ("persistent_fx.cu", "dslash_fx.cuh", "fx.cuh", "warp_sum.cuh"))}
 
 
 def _peaks():
@@ -1047,10 +1047,10 @@ def main():
         return
 
     peaks = _peaks()
-    fam_names = {gs.GS_PROF_STENCIL_F64: "k_dslash_f64 (Wilson stencil on label ranges, FP64)",
-                 gs.GS_PROF_SOLVER_F64: "k_bicg_persistent_f64 (whole inner BiCGStab solve in one "
-                                         "cooperative launch: two D_rr stencils + vector updates per "
-                                         "iteration, FP64)"}
+    fam_names = {gs.GS_PROF_STENCIL_F64: "k_dslash_fx (Wilson stencil on label ranges, FP64 in block fixed point)",
+                 gs.GS_PROF_SOLVER_F64: "k_bicg_persistent_fx (whole inner BiCGStab solve in one "
+                                         "cooperative launch: two D_rr stencils in block fixed point + "
+                                         "FP64 vector updates per iteration)"}
     dom = max(prof, key=lambda fam: prof[fam]["union_ms"])
 
     def fam_view(p):

@@ -170,10 +170,11 @@ enum { GS_OPT_STENCIL_VARIANT = 1, GS_OPT_INNER_KERNEL = 2, GS_OPT_NET_KERNEL = 
  * solver kernels of this problem use while schur_solve_batched runs several
  * solves at once (the caller then keeps their sum within what the GPU holds
  * at once); 0 = granted at each launch by the call's block ledger (the
- * default): on rest sets of at most 16384 sites one pass over the set (FP64:
- * one round of 32-site tiles; FP32 / BF16: about 96 sites per block), above
- * that an even share of the co-resident blocks among the running solves,
- * never more than the other solves leave free.
+ * default): FP64 inner solves of a call whose rest sets all have at most 32
+ * sites per SM take a block per 32-site tile, others an even share of the
+ * co-resident blocks among the running solves; FP32 / BF16 about 96 sites per
+ * block on rest sets of at most 16384 sites, an even share above; never more
+ * than the other solves leave free.
  * GS_OPT_BATCH_LANES (read from the first problem's context): how many solves
  * schur_solve_batched runs at once, 1 .. 64; 0 = four (the default). */
 gs_status gs_set_option(gs_ctx* ctx, int option, int value);
@@ -296,11 +297,11 @@ gs_status gs_profile_read(gs_ctx* ctx, int family, gs_kernel_profile* out);
 gs_status gs_profile_timeline(gs_ctx* ctx, int family, double* out, int cap, int* n_out);
 /* SM clock cycles that block 0 of the persistent FP64 BiCGStab spent in each
  * phase of its iterations while profiling was on (summed over launches):
- * out[3 s + 0] = work of step s (s = 0: v = D p and <rhat, v>; 1: s = r - a v
- * and ||s||^2; 2: t = D s, <t, s>, <t, t>, <rhat, t>; 3: the x, r and p
- * updates and ||r||^2; 4: unused, 0), out[3 s + 1] = its grid barrier,
- * out[3 s + 2] = the reduction of the per-block partials and the scalar
- * algebra after it.  n >= 15.  A diagnostic of where an iteration's time
+ * out[3 s + 0] = work of step s (s = 0: v = D p and <rhat, v>; 1: s = r - a v;
+ * 2: t = D s and the dots with t, s and rhat; 3: the r and p updates; 4:
+ * unused, 0), out[3 s + 1] = the wait for the other blocks' partial sums,
+ * out[3 s + 2] = their total and the scalar algebra after it (steps 1 and 3
+ * end in no reduction: 0 there).  n >= 15.  A diagnostic of where an iteration's time
  * goes; synchronises. */
 gs_status gs_profile_phases(gs_ctx* ctx, double* out, int n);
 

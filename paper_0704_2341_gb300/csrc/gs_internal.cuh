@@ -188,7 +188,8 @@ struct gs_ctx;
 
 namespace gs {
 // The blocks of the persistent solver kernels of one schur_solve_batched
-// call.  In one call those blocks all have one size, so they are interchangeable and the GPU holds per_sm x SMs of them at once.
+// call.  In one call those blocks all have one size, so they are
+// interchangeable and the GPU holds per_sm x SMs of them at once.
 // held[] records, per running solve, the blocks its kernel may have in
 // flight: its last grid (its previous kernel has finished before it launches
 // again), or nothing before its first launch.  A grid is granted only from

@@ -921,10 +921,13 @@ static void gradw_dispatch(int C, int cin, int cout, const float2* in, const flo
 static gs_status net_prepare(gs_ctx* c, gs_net* nt, int B = 1) {
     const int64_t V = c->V;
     if (nt->capV < V || nt->capB < B) {
-        for (auto& a : nt->act) cudaFree(a);
-        for (auto& a : nt->gact) cudaFree(a);
-        cudaFree(nt->U32);
-        nt->U32 = nullptr;
+        auto drop = [](auto& a) {
+            cudaFree(a);
+            a = nullptr;       // an allocation below may fail: nothing is freed twice
+        };
+        for (auto& a : nt->act) drop(a);
+        for (auto& a : nt->gact) drop(a);
+        drop(nt->U32);
         nt->U32_src = nullptr;
         const size_t big = (size_t)B * V * 4 * nt->C * 3 * sizeof(float2);
         const size_t sm = (size_t)B * V * 12 * sizeof(float2);
