@@ -1100,7 +1100,7 @@ def main():
         "config": {"workload": WORKLOAD, "solves_per_step": len(PERMS),
                    "form": "plain FP64; the four permutations' solves at once (schur_solve_batched: one "
                            "context and stream per permutation, each solve's persistent kernels granted "
-                           "one round of 32-site tiles, 120 or 64 of the 456 co-resident blocks, by the "
+                           "a block per 32-site tile, 120 or 64 of the 304 co-resident blocks, by the "
                            "call's block ledger)",
                    "l2": "flushed between steps (256 MiB write)",
                    "parallelism": "replicas" if world > 1 else "single GPU",

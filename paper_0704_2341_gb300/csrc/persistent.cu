@@ -656,12 +656,12 @@ __global__ void __launch_bounds__(kPThreads) k_selftest_grid_timeout(GridSync g,
 
 // co-resident grid for a cooperative launch on a set of rest_sites sites: at
 // most `want` blocks.  Inside schur_solve_batched (no GS_OPT_COOP_BLOCKS) the
-// grid comes from the call's block ledger: on a small rest set a kernel that
-// passes `round` (the blocks for one pass over the set) asks for exactly
-// that -- on 8^4 the four permutations' FP64 solves take 120 + 64 + 120 + 64
-// of the 456 co-resident blocks, one tile round per stencil phase each
-// (45.0 solves/s against 40.2 with 76 blocks each); otherwise it asks for its
-// share of the GPU while n solves run (two blocks per SM on small sets, all
+// grid comes from the call's block ledger (only the low-precision solver gets here
+// with one: the FP64 solver of a batched call is persistent_fx.cu's): on a small
+// rest set a kernel that passes `round` (the blocks for one pass over the set)
+// asks for exactly that -- FP32 inner solves on 8^4, 96 sites per block, 84.9
+// solves/s against 75.8 with 76 blocks each; otherwise it asks for its share
+// of the GPU while n solves run (two blocks per SM on small sets, all
 // co-resident blocks on large ones).
 template <class K>
 static int coop_grid(gs_ctx* c, K kernel, int64_t want, int64_t rest_sites, int64_t round = 0) {
