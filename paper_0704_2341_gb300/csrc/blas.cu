@@ -31,13 +31,13 @@ __device__ __forceinline__ double sum_of_block(const double* sm) {
     double x[kBlas / 32];
 #pragma unroll
     for (int m = 0; m < kBlas / 32; ++m) x[m] = sm[m * 32 + lane];
-    return warp_sum<kBlas / 32>(x);
+    return warp_sum<kBlas / 32, true>(x);
 }
 __device__ __forceinline__ double sum_of_partials(const double* part, int64_t ld, int n) {
     const int lane = threadIdx.x & 31;
     if (n <= 32) {
         const double x[1] = {lane < n ? __ldcg(part + lane * ld) : 0.0};
-        return warp_sum<1>(x);
+        return warp_sum<1, true>(x);
     }
     double t = 0.0;
     for (int b0 = 0; b0 < n; b0 += 32 * 10) {
@@ -47,7 +47,7 @@ __device__ __forceinline__ double sum_of_partials(const double* part, int64_t ld
             const int b = b0 + 32 * m + lane;
             x[m] = b < n ? __ldcg(part + b * ld) : 0.0;
         }
-        t += warp_sum<10>(x);
+        t += warp_sum<10, true>(x);
     }
     return t;
 }

@@ -154,8 +154,8 @@ __global__ void __launch_bounds__(kBsrThreads) k_bsr_apply(BsrArgs a, BsrDots d)
         constexpr int NV = DOTS == BSR_OMEGA ? 3 : 2;
         if (tid < 32) {
             const double x0[1] = {e0}, x1[1] = {e1}, x2[1] = {e2};
-            const double t0 = warp_sum<1>(x0), t1 = warp_sum<1>(x1);
-            const double t2 = NV == 3 ? warp_sum<1>(x2) : 0.0;
+            const double t0 = warp_sum<1, true>(x0), t1 = warp_sum<1, true>(x1);
+            const double t2 = NV == 3 ? warp_sum<1, true>(x2) : 0.0;
             if (lane == 0) {
                 double* q = d.red.partial + (int64_t)blockIdx.x * kMaxRedVals;
                 q[0] = t0;
@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(kBsrThreads) k_bsr_apply(BsrArgs a, BsrDots d)
                     const unsigned b = b0 + 32 * m + lane;
                     x[m] = b < gridDim.x ? __ldcg(d.red.partial + (int64_t)b * kMaxRedVals + q) : 0.0;
                 }
-                t += warp_sum<8>(x);
+                t += warp_sum<8, true>(x);
             }
             if (lane == 0) tot[q] = t;
         }

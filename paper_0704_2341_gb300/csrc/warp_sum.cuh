@@ -19,8 +19,10 @@ __device__ __forceinline__ long long warp_add(long long m) {
 // added as 54-bit integers under the largest one's exponent: the error is at
 // most 2^-55 of the largest value per term, below that of a double-precision
 // tree, whose partial sums round at 2^-53.  Sums out of the usual range take
-// that tree.
-template <int N>
+// that tree; with REFINE also sums that cancel to nothing, where it still has the
+// small terms' last bits: a host-driven Krylov method takes an exact zero for a
+// breakdown (one of 16 runs of 3000 steps that do not converge met rho = 0).
+template <int N, bool REFINE = false>
 __device__ __forceinline__ double warp_sum(const double (&x)[N]) {
     static_assert(N <= 16, "the integer sum would overflow");
     int E = 0;
@@ -28,19 +30,20 @@ __device__ __forceinline__ double warp_sum(const double (&x)[N]) {
     for (int k = 0; k < N; ++k) E = max(E, fx_exponent((unsigned)__double2hiint(x[k])));
     E = __reduce_max_sync(0xffffffffu, E);
     if (E == 0) return 0.0;
-    if (E < kFxMinExp || E > 1900) {
-        double s = 0.0;
+    if (E >= kFxMinExp && E <= 1900) {
+        long long m = 0;
 #pragma unroll
-        for (int k = 0; k < N; ++k) s += x[k];
-#pragma unroll 1
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        return s;
+        for (int k = 0; k < N; ++k)
+            m += fx_from_bits((unsigned)__double2hiint(x[k]), (unsigned)__double2loint(x[k]), E + 6);
+        m = warp_add(m);
+        if (!REFINE || m != 0) return fx_to_double(m, E + 3);
     }
-    long long m = 0;
+    double s = 0.0;
 #pragma unroll
-    for (int k = 0; k < N; ++k)
-        m += fx_from_bits((unsigned)__double2hiint(x[k]), (unsigned)__double2loint(x[k]), E + 6);
-    return fx_to_double(warp_add(m), E + 3);
+    for (int k = 0; k < N; ++k) s += x[k];
+#pragma unroll 1
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    return s;
 }
 
 // The same for floats (24 of 54 bits are the largest value's own).
