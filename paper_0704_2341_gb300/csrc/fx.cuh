@@ -14,10 +14,14 @@
 // double is 4.7e-17; the double-precision kernel, whose hop arithmetic rounds some
 // sixty times at 2^-53 of its partial sums, is 9.3e-17 off.
 //
-// Ranges: |u 2^61| <= 2^60 x 1.01 (links are checked when they are packed),
-// |x 2^60 / 2^e| < 2^60, a projected component below 2^61.  A row is six products
-// below 1.01 2^57, its middle sum twelve below 1.01 2^59, eight hops below
-// 2^62.7: nothing overflows 63 bits, unitary links or not.
+// Ranges: |u 2^61| <= 2^60 x 1.01, |x 2^60 / 2^e| < 2^60, a projected component
+// h below 2^61.  A row's middle sum has six terms u.hi h.lo, below 2^60 |u| each, and
+// six u.lo h.hi, below 2^60 each: with R = the sum of |re| + |im| over a row (forward hop)
+// or a column (backward hop) of the link it stays below (R + 6) 2^60, so R <= kFxRowMax
+// = 1.9 keeps it below 7.9 2^60 < 2^63.  (R is at most sqrt 6 / 2 = 1.23 for a unitary U; six entries
+// at the limit of kFxLinkMax alone would reach 9.03 2^60.)  The row's products are then below
+// 1.9 2^58, and eight hops below 2^62.  Entries and R are checked when the links are
+// packed; a field that fails either check is done in double precision.
 #pragma once
 
 #include <stdint.h>
@@ -30,6 +34,7 @@ constexpr int kFxZero = 0;        // exponent word of a site whose components ar
 constexpr int kFxBad = -1;        // a component is not finite, or the site's scale is out of range
 constexpr int kFxMinExp = 128, kFxMaxExp = 1920;   // accepted biased exponents of a site's largest component
 constexpr double kFxLinkMax = 0.505;               // largest |re|, |im| of -1/2 U (0.5 for a unitary U)
+constexpr double kFxRowMax = 1.9;                  // largest sum of |re| + |im| over a row or column of -1/2 U
 
 struct FxLimb {
     int hi, lo;
@@ -38,6 +43,18 @@ struct FxLimb {
 __host__ __device__ __forceinline__ FxLimb fx_split(long long v) {
     const unsigned lo = (unsigned)v, hi = (unsigned)((unsigned long long)v >> 32);
     return FxLimb{(int)(hi + (lo >> 31)), (int)lo};
+}
+
+// Whether the three entries p[0], p[ld], p[2 ld] of a packed link, limbs (re.lo, re.hi,
+// im.lo, im.hi), have a sum of |re| + |im| within kFxRowMax.
+__host__ __device__ __forceinline__ bool fx_row_fits(const int4* p, int ld) {
+    long long sum = 0;
+    for (int c = 0; c < 3; ++c) {
+        const int4 u = p[c * ld];
+        const long long re = (long long)u.y * 4294967296ll + u.x, im = (long long)u.w * 4294967296ll + u.z;
+        sum += (re < 0 ? -re : re) + (im < 0 ? -im : im);
+    }
+    return sum <= (long long)(kFxRowMax * 2305843009213693952.0);     // 2^61
 }
 
 // accumulator of products: hh counts 2^64 units, md 2^32 units

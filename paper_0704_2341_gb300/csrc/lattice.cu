@@ -132,8 +132,8 @@ __global__ void k_count_hops(int64_t V, int64_t nb, const int2* __restrict__ nbr
 // links[j][mu][k] = -1/2 * U[perm[j]][mu][k]  (the factor is exact in binary),
 // and the same in fixed point, in groups of 32 labels (fx_index): a block turns
 // 32 sites around in shared memory so that both arrays are written in whole
-// lines.  *flag = 1 if an entry does not fit fixed point (the stencils then
-// use the double-precision links).
+// lines.  *flag = 1 if an entry, or the sum of a row or a column, does not fit
+// fixed point (the stencils then use the double-precision links).
 __global__ void __launch_bounds__(256) k_pack_links(int64_t V, const int32_t* __restrict__ perm,
                                                     const double2* __restrict__ U, double2* __restrict__ links,
                                                     int4* __restrict__ fx, int* __restrict__ flag) {
@@ -155,6 +155,11 @@ __global__ void __launch_bounds__(256) k_pack_links(int64_t V, const int32_t* __
         for (int i = threadIdx.x; i < 36 * 32; i += 256) {
             const int k = i >> 5, site = i & 31;
             if (site < n) fx[base * 36 + i] = sm[site][k];
+        }
+        // forward hops take the rows of a link, backward hops its columns
+        for (int i = threadIdx.x; i < 24 * 32; i += 256) {
+            const int site = i & 31, q = i >> 5, mu = q / 6, r = q - 6 * mu;
+            if (site < n && !fx_row_fits(sm[site] + mu * 9 + (r < 3 ? 3 * r : r - 3), r < 3 ? 1 : 3)) atomicExch(flag, 1);
         }
         __syncthreads();
     }
