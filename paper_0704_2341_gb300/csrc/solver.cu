@@ -156,7 +156,10 @@ gs_status inner_solve_f64(gs_ctx* c, const Plan* p, const double2* t, double2* z
         // the whole solve in one cooperative launch (persistent_fx.cu); a field
         // or right-hand side that fixed point cannot hold goes to the
         // double-precision kernel (persistent.cu), or inside a batched call,
-        // whose block ledger counts blocks of one size, to the per-phase launches
+        // whose block ledger counts blocks of one size, to the per-phase launches.
+        // So does a solve that ended on a zero inner product: the integer sums
+        // give an exact zero where the large terms cancel below 2^-54 of the
+        // largest, and only sums in double precision tell that from a breakdown.
         int slot = -1;
         if (c->prof.on && (s = prof_begin(c, &slot)) != GS_OK) return s;
         auto finished = [&]() -> gs_status {
@@ -168,7 +171,7 @@ gs_status inner_solve_f64(gs_ctx* c, const Plan* p, const double2* t, double2* z
         s = persistent_bicg_fx(c, p, k1, t, z, w, o.inner_tol, o.inner_max_iter);
         if (s != GS_OK || (s = finished()) != GS_OK) return s;
         ledger_release(c);
-        if (pub->status == kFxUnfit) {
+        if (pub->status == kFxUnfit || pub->status == GS_BREAKDOWN) {
             if (c->ledger) kernel = 1;
             else {
                 s = persistent_bicg_f64(c, k1, k3, t, z, w, n, o.inner_tol, o.inner_max_iter);

@@ -21,7 +21,9 @@ __device__ __forceinline__ long long warp_add(long long m) {
 // tree, whose partial sums round at 2^-53.  Sums out of the usual range take
 // that tree; with REFINE also sums that cancel to nothing, where it still has the
 // small terms' last bits: a host-driven Krylov method takes an exact zero for a
-// breakdown (one of 16 runs of 3000 steps that do not converge met rho = 0).
+// breakdown (one of 16 runs of 3000 steps that do not converge met rho = 0).  The
+// persistent FP64 solver goes without it: its host takes a solve that ended on a zero
+// again in double precision.
 template <int N, bool REFINE = false>
 __device__ __forceinline__ double warp_sum(const double (&x)[N]) {
     static_assert(N <= 16, "the integer sum would overflow");

@@ -59,3 +59,26 @@ def test_links_with_large_rows(env, entries):
     x = np.repeat((1 + 1j) * 0.9 * rng.uniform(0.99, 1.01, (V, 1)), 12, 1)
     y, ref = _both(env, dims, -0.35, U, x)
     assert np.abs(y - ref).max() <= 2 * 61 * 2.0 ** -53 * 38.3 * np.sqrt(2) * np.abs(x).max()
+
+
+def test_a_dot_that_cancels_is_not_a_breakdown(env):
+    """<b, D_rr b> of terms -1/2, -1/2, 1/2, 1/2 and 124 of 0.9 x 2^-55: the small ones vanish
+    beside the large ones in the fixed-point sums, but the dot is not zero.  m0 = -4 takes
+    the diagonal away; the only links join the pairs x3 = 0, 1 and 2, 3."""
+    torch, gs = env
+    dims = (4, 4, 4, 4)
+    V = li.volume(dims)
+    s = np.arange(V)
+    x0, x3, first = s % 4, s // 64, (s % 64) == 1        # `first`: the line of the large terms
+    U = np.zeros((V, 4, 3, 3), complex)
+    up = x3 % 2 == 0
+    U[up, 3] = -np.eye(3)
+    U[first & (x3 == 0), 3] = np.eye(3)
+    full = np.zeros((V, 12), complex)
+    full[:, 0] = np.where(first, 1.0, np.where(up, 1.0, 0.9) * 2.0 ** -27)
+    b = to_dev(full[x0 % 2 == 1], torch)                 # Type II, direction 0: the rest set, in order
+    ctx = _ctx(gs, torch, dims, -4.0, U)
+    z = torch.empty_like(b)
+    st = ctx.solve_rr(2, 0, 0, b, z, gs.gs_default_opts(inner_max_iter=1), allow=(gs.GS_MAXITER,))
+    assert st.status == gs.GS_MAXITER and st.inner_iters == 1
+    ctx.close()
