@@ -82,3 +82,23 @@ def test_a_dot_that_cancels_is_not_a_breakdown(env):
     st = ctx.solve_rr(2, 0, 0, b, z, gs.gs_default_opts(inner_max_iter=1), allow=(gs.GS_MAXITER,))
     assert st.status == gs.GS_MAXITER and st.inner_iters == 1
     ctx.close()
+
+
+# Powers of two change no rounding: the solve is the same, step by step, and its result the scaled one.
+@pytest.mark.parametrize("dims,t", [((4, 4, 4, 2), 1), ((8, 8, 8, 10), 1), ((9, 10, 11, 12), 2)])
+@pytest.mark.parametrize("power", [-200, -130, -100, 100, 130, 200])
+def test_rest_solve_at_any_scale(env, dims, t, power):
+    torch, gs = env
+    rng = np.random.default_rng(12)
+    mu = 1 if dims[0] % 2 else 0
+    V = li.volume(dims)
+    nr = V - (V // 16 if t == 1 else V // 2)
+    b = to_dev(rng.standard_normal((nr, 12)) + 1j * rng.standard_normal((nr, 12)), torch)
+    ctx = _ctx(gs, torch, dims, 0.1, li.random_gauge(dims, 0.3, 13))
+    o = gs.gs_default_opts(inner_tol=1e-13)
+    z1, z2 = torch.empty_like(b), torch.empty_like(b)
+    one = ctx.solve_rr(t, mu, 0, b, z1, o)
+    two = ctx.solve_rr(t, mu, 0, b * 2.0 ** power, z2, o)
+    assert two.inner_iters == one.inner_iters
+    assert torch.equal(z2, z1 * 2.0 ** power)
+    ctx.close()
