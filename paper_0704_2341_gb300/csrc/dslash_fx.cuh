@@ -45,6 +45,10 @@ struct FxOperands {
 // X_mu pairs spins 0, 1 with 3, 2 (mu < 2) or 2, 3
 __device__ __forceinline__ int fx_partner(int w, int s) { return ((w < 8) != (s != 0)) ? 9 : 6; }
 
+// Mantissas and exponents are plain loads: the kernel that writes them may still be
+// running when this one starts (programmatic launch), so they are not constant
+// for this kernel's lifetime, as __ldg would have it, and only a plain load stays
+// behind griddepcontrol.wait.
 template <int NS, bool CG>
 __device__ __forceinline__ void fx_load_spinor(const StencilArgs& a, int w, int in, FxOperands<NS>& o) {
     const longlong2* p = a.fxm + fx_index(in, kSiteC);
@@ -55,8 +59,8 @@ __device__ __forceinline__ void fx_load_spinor(const StencilArgs& a, int w, int 
         const longlong2* pq = p + fx_partner(w, s) * 32;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            o.s[k][c] = CG ? __ldcg(ps + c * 32) : __ldg(ps + c * 32);
-            o.q[k][c] = CG ? __ldcg(pq + c * 32) : __ldg(pq + c * 32);
+            o.s[k][c] = CG ? __ldcg(ps + c * 32) : ps[c * 32];
+            o.q[k][c] = CG ? __ldcg(pq + c * 32) : pq[c * 32];
         }
     }
 }
@@ -184,7 +188,7 @@ template <bool CG>
 __device__ __forceinline__ int fx_site(const StencilArgs& a, int l, unsigned& i) {
     i = l < 0 ? 0xffffffffu : (unsigned)l - (unsigned)a.a0;   // labels below the range wrap above it
     if (i >= (unsigned)a.fxn) return kFxZero;
-    return CG ? __ldcg(a.fxe + i) : __ldg(a.fxe + i);
+    return CG ? __ldcg(a.fxe + i) : a.fxe[i];
 }
 
 // One tile of ts <= 32 output sites from base, l = fx_label of this tile.

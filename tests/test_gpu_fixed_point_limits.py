@@ -102,3 +102,27 @@ def test_rest_solve_at_any_scale(env, dims, t, power):
     assert two.inner_iters == one.inner_iters
     assert torch.equal(z2, z1 * 2.0 ** power)
     ctx.close()
+
+
+@pytest.mark.parametrize("dims", [(8, 8, 8, 8), (8, 10, 8, 24)])
+def test_applications_back_to_back(env, dims):
+    """The conversion of an input and the stencil overlap at the edges: in a row of
+    applications to inputs of different scale each result is that of its own input."""
+    torch, gs = env
+    rng = np.random.default_rng(14)
+    V = li.volume(dims)
+    ctx = _ctx(gs, torch, dims, -0.35, li.random_gauge(dims, 0.3, 15))
+    xs = [to_dev(s * (rng.standard_normal((V, 12)) + 1j * rng.standard_normal((V, 12))), torch)
+          for s in (1.0, 1e-9, 1e9)]
+    alone = []
+    for x in xs:
+        y = torch.empty_like(x)
+        ctx.wilson_apply(x, y)
+        torch.cuda.synchronize()
+        alone.append(y)
+    ys = [torch.full_like(xs[0], float("nan")) for _ in range(60)]
+    for k, y in enumerate(ys):
+        ctx.wilson_apply(xs[k % 3], y)
+    torch.cuda.synchronize()
+    assert all(torch.equal(y, alone[k % 3]) for k, y in enumerate(ys))
+    ctx.close()
