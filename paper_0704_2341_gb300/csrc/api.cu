@@ -322,6 +322,7 @@ gs_status wilson_apply(gs_ctx* c, const void* x_dev, void* y_dev) {
     a.plan = p;
     a.nbr = p->nbr;
     a.links = p->links;
+    a.keep_weak = 1;
     return launch_stencil_f64(c, a);
 }
 

@@ -55,10 +55,11 @@ __global__ void __launch_bounds__(kThreads) k_fx_pack(const double2* __restrict_
     }
 }
 
-template <int EPI, int NS>
+template <int EPI, int NS, bool KEEP>
 __global__ void __launch_bounds__(kFxThreads<NS>, NS) k_dslash_fx(const __grid_constant__ StencilArgs a) {
     __shared__ FxShared sm;
     __shared__ int sE[8][kSitesPerBlock];
+    __shared__ unsigned redo[KEEP ? kFxRedoWords : 1];
     const int l = fx_label(a, (int64_t)blockIdx.x * kSitesPerBlock, kSitesPerBlock, (threadIdx.x >> 5) * NS);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const bool skip = a.st != nullptr && a.st->done;
@@ -66,7 +67,7 @@ __global__ void __launch_bounds__(kFxThreads<NS>, NS) k_dslash_fx(const __grid_c
     if (skip) return;
     const bool links_bad = __ldg(a.fxflag) != 0;
     double e[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    fx_stencil<EPI, false, NS>(a, kSitesPerBlock, links_bad, sm, sE, l, e);
+    fx_stencil<EPI, false, NS, KEEP>(a, kSitesPerBlock, links_bad, sm, sE, redo, l, e);
     stencil_finish<EPI, kFxThreads<NS>>(a, e);
 }
 
@@ -76,12 +77,16 @@ __global__ void __launch_bounds__(kFxThreads<NS>, NS) k_dslash_fx(const __grid_c
 // against 0.61).
 template <int NS>
 cudaError_t launch_fx(const StencilArgs& a, cudaLaunchConfig_t cfg, int grid, int sms) {
-    cfg.gridDim = dim3(grid < NS * sms ? grid : NS * sms);
+    const int64_t tiles = (a.n_out + kSitesPerBlock - 1) / kSitesPerBlock;
+    const int least = (int)((tiles + 32 * kFxRedoWords - 1) / (32 * kFxRedoWords));   // blocks whose tiles fit `redo`
+    const int most = NS * sms > least ? NS * sms : least;
+    cfg.gridDim = dim3(grid < most ? grid : most);
     cfg.blockDim = dim3(kFxThreads<NS>);
     switch (a.epi) {
-        case EPI_NONE: return cudaLaunchKernelEx(&cfg, k_dslash_fx<EPI_NONE, NS>, a);
-        case EPI_DOT_RHAT_V: return cudaLaunchKernelEx(&cfg, k_dslash_fx<EPI_DOT_RHAT_V, NS>, a);
-        default: return cudaLaunchKernelEx(&cfg, k_dslash_fx<EPI_DOT_TS, NS>, a);
+        case EPI_NONE:
+            return cudaLaunchKernelEx(&cfg, a.keep_weak ? k_dslash_fx<EPI_NONE, NS, true> : k_dslash_fx<EPI_NONE, NS, false>, a);
+        case EPI_DOT_RHAT_V: return cudaLaunchKernelEx(&cfg, k_dslash_fx<EPI_DOT_RHAT_V, NS, false>, a);
+        default: return cudaLaunchKernelEx(&cfg, k_dslash_fx<EPI_DOT_TS, NS, false>, a);
     }
 }
 

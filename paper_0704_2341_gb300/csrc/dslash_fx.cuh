@@ -173,6 +173,29 @@ __device__ __forceinline__ I2 fx_sum(const FxShared& sm, int site, int spin, int
     return fx_add_i(fx_sub_i(d[3] - d[1], d[0]), d[2]);               // -i d0 - d1 + i d2 + d3
 }
 
+// Fixed point resolves 2^-57 of the largest input component around a site, double
+// precision 2^-53 of the terms of each component: a component whose terms are all
+// small beside that maximum (a weak spin component; a weak colour where the links
+// are near the identity) would lose digits that double precision keeps.  Such a
+// component is `weak`: every hop's contribution is below 2^-k of the scale 2^E, k by
+// the number of hops in range, and its tile is done in double precision.  A tile
+// in double precision takes some 15 us, so the lines lie where Gaussian spinors
+// meet them in less than 1e-8 of the components: |re| and |im| of a contribution are
+// both below 2^-8 with probability 3e-4, 2^-10 2e-5, 2^-16 5e-9.
+// Contributions that are zero because their inputs are (point sources and probes)
+// are exact in fixed point.
+constexpr int kFxWeak1 = 16, kFxWeak2 = 10, kFxWeak = 8;     // k for one hop, two, more
+
+__device__ __forceinline__ int fx_weak_bits(int hops) {
+    return 57 - (hops > 2 ? kFxWeak : hops > 1 ? kFxWeak2 : kFxWeak1);
+}
+// bits 32.. of the magnitude
+__device__ __forceinline__ int fx_top(long long v) {
+    const int hi = (int)(v >> 32);
+    return hi ^ (hi >> 31);
+}
+constexpr int kFxWeakSum = 1 << (57 - kFxWeak + 3 - 32);     // a sum of up to eight such contributions stays below
+
 // The label of the tile's site `lane`'s neighbour that hop w reads (-1: no such
 // site); fetched a tile ahead of its use.
 __device__ __forceinline__ int fx_label(const StencilArgs& a, int64_t base, int ts, int w) {
@@ -191,12 +214,46 @@ __device__ __forceinline__ int fx_site(const StencilArgs& a, int l, unsigned& i)
     return CG ? __ldcg(a.fxe + i) : a.fxe[i];
 }
 
+// Whether the inputs of a spin component's hops are zero: what fixed point then gives
+// for it, zero, is exact.  j: the site's label.
+__device__ __forceinline__ bool fx_silent(const StencilArgs& a, int64_t j, int spin) {
+#pragma unroll 1
+    for (int q = 0; q < 8; ++q) {
+        const int2 n = __ldg(a.nbr + j * 4 + (q >> 1));
+        const int64_t l = (q & 1) ? n.y : n.x;
+        const double2* p = l >= a.a0 && l < a.a1 ? a.inA + (l - a.a0) * kSiteC
+                           : l >= a.a1 && l < a.b1 ? a.inB + (l - a.a1) * kSiteC : nullptr;
+        if (!p) continue;
+        const int up = spin < 2 ? spin : q < 4 ? 3 - spin : spin - 2;       // upper spin of the hop's row, and its partner
+        const int lo = q < 4 ? 3 - up : 2 + up;
+#pragma unroll 1
+        for (int c = 0; c < 3; ++c) {
+            const double2 s = __ldg(p + 3 * up + c), t = __ldg(p + 3 * lo + c);
+            if (s.x != 0.0 || s.y != 0.0 || t.x != 0.0 || t.y != 0.0) return false;
+        }
+    }
+    return true;
+}
+__device__ __forceinline__ bool fx_weak(const FxShared& sm, const int (&sE)[8][kSitesPerBlock], int site, int spin,
+                                        int c) {
+    int hops = 0, top = 0;
+    const int w01 = spin < 2 ? spin : 3 - spin, w23 = spin & 1;      // row within a direction: mu < 2, mu >= 2
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const longlong2 g = sm.hop[2 * q + (q < 4 ? w01 : w23)][site][c];
+        top |= fx_top(g.x) | fx_top(g.y);
+        hops += sE[q][site] > 0;
+    }
+    return hops > 0 && top < 1 << (fx_weak_bits(hops) - 32);
+}
+
 // One tile of ts <= 32 output sites from base, l = fx_label of this tile.
 // Phase 1: a warp per hop (and spin component).  Phase 2: three warps per spin
 // component, a thread one complex output: sum of the hops, conversion,
-// diagonal, addend and the epilogue dots.  Returns true, with nothing written,
-// if an input site of the tile does not fit fixed point.
-template <int EPI, bool CG, int NS>
+// diagonal, addend and the epilogue dots.  Returns true if the tile has to be done
+// in double precision: an input site does not fit fixed point (nothing is written), or
+// with KEEP a component is weak.  The output is not the addend.
+template <int EPI, bool CG, int NS, bool KEEP>
 __device__ __forceinline__ bool fx_tile(const StencilArgs& a, int64_t base, int ts, int l, FxShared& sm,
                                         int (&sE)[8][kSitesPerBlock], double (&e)[5]) {
     const int warp = threadIdx.x >> 5;
@@ -227,6 +284,7 @@ __device__ __forceinline__ bool fx_tile(const StencilArgs& a, int64_t base, int 
         }
     }
     if (__syncthreads_or(bad)) return true;
+    unsigned weak = 0;         // bit per component of this thread
     for (int v = warp; v < 12; v += kFxThreads<NS> / 32) {
         const int spin = v / 3;
         const int i = (v - 3 * spin) * 32 + lane;
@@ -237,6 +295,7 @@ __device__ __forceinline__ bool fx_tile(const StencilArgs& a, int64_t base, int 
 #pragma unroll
         for (int q = 0; q < 8; ++q) E = max(E, sE[q][site]);
         const int64_t j = a.o0 + base + site;
+        if (KEEP && (fx_top(t.x) | fx_top(t.y)) < kFxWeakSum && fx_weak(sm, sE, site, spin, c)) weak |= 1u << v;
         const int k = 3 * spin + c;
         const double2* self = nullptr;
         if (j >= a.a0 && j < a.a1) self = a.inA + (j - a.a0) * kSiteC + k;
@@ -260,23 +319,56 @@ __device__ __forceinline__ bool fx_tile(const StencilArgs& a, int64_t base, int 
         a.out[o] = make_double2(re, im);
         stencil_dots<EPI, CG>(a, o, re, im, e);
     }
+    if (KEEP) {
+        if (!__syncthreads_or(weak)) return false;
+        bool keep = false;
+#pragma unroll 1
+        for (int v = warp; v < 12; v += kFxThreads<NS> / 32)
+            if (weak >> v & 1u) keep |= !fx_silent(a, a.o0 + base + ((v % 3) * 32 + lane) / 3, v / 3);
+        return __syncthreads_or(keep);
+    }
     __syncthreads();
     return false;
 }
 
+// Tiles of a block that double precision has to do, a bit each (V < 2^31 / 12 sites in
+// tiles of 32 over 2 blocks an SM: at most 18 400 tiles a block on 152 SMs).
+constexpr int kFxRedoWords = 640;
+
 // The block's tiles of the stencil; those that fixed point cannot hold (all of
 // them when a link does not fit) are done in double precision afterwards, so
-// that the rare path costs the common one no registers.
-template <int EPI, bool CG, int NS>
+// that the rare path costs the common one no registers.  With KEEP `redo` holds them, as
+// the hops' sums are gone by then.
+template <int EPI, bool CG, int NS, bool KEEP>
 __device__ __forceinline__ void fx_stencil(const StencilArgs& a, int ts, bool links_bad, FxShared& sm,
-                                           int (&sE)[8][kSitesPerBlock], int l, double (&e)[5]) {
+                                           int (&sE)[8][kSitesPerBlock], unsigned* redo, int l, double (&e)[5]) {
     const int64_t step = (int64_t)gridDim.x * ts;
     const int w = (threadIdx.x >> 5) * NS;
     bool any = links_bad;
+    if constexpr (KEEP) {
+        for (int i = threadIdx.x; i < kFxRedoWords; i += kFxThreads<NS>) redo[i] = links_bad ? ~0u : 0u;
+        int tile = 0;
+        if (!links_bad)
+            for (int64_t base = (int64_t)blockIdx.x * ts; base < a.n_out; base += step, ++tile) {
+                const int next = fx_label(a, base + step, ts, w);
+                if (fx_tile<EPI, CG, NS, true>(a, base, ts, l, sm, sE, e)) {
+                    any = true;
+                    if (threadIdx.x == 0) redo[tile >> 5] |= 1u << (tile & 31);
+                }
+                l = next;
+            }
+        if (any) {
+            __syncthreads();
+            tile = 0;
+            for (int64_t base = (int64_t)blockIdx.x * ts; base < a.n_out; base += step, ++tile)
+                if (redo[tile >> 5] >> (tile & 31) & 1u) f64_tile<EPI, CG>(a, base, ts, sm.f64, e);
+        }
+        return;
+    }
     if (!links_bad)
         for (int64_t base = (int64_t)blockIdx.x * ts; base < a.n_out; base += step) {
             const int next = fx_label(a, base + step, ts, w);
-            any |= fx_tile<EPI, CG, NS>(a, base, ts, l, sm, sE, e);
+            any |= fx_tile<EPI, CG, NS, false>(a, base, ts, l, sm, sE, e);
             l = next;
         }
     if (any)

@@ -12,7 +12,10 @@
 // around the output site.  Against a 64-bit-mantissa reference of D x (8^4,
 // Gaussian x) the relative error is 5.9e-17, of which rounding the result to
 // double is 4.7e-17; the double-precision kernel, whose hop arithmetic rounds some
-// sixty times at 2^-53 of its partial sums, is 9.3e-17 off.
+// sixty times at 2^-53 of its partial sums, is 9.3e-17 off.  That holds for vectors
+// whose components are of like size; where one is small beside its neighbours its
+// digits below the unit are lost, so wilson_apply sends such tiles to double
+// precision (fx_weak, dslash_fx.cuh).
 //
 // Ranges: |u 2^61| <= 2^60 x 1.01, |x 2^60 / 2^e| < 2^60, a projected component
 // h below 2^61.  A row's middle sum has six terms u.hi h.lo, below 2^60 |u| each, and

@@ -355,6 +355,8 @@ struct StencilArgs {
     int64_t fxn;
     const int4* fxl;
     const int* fxflag;
+    int keep_weak;           // each component as accurate as its own terms (fx_weak): wilson_apply's result;
+                             // the other callers' vectors matter by their norms
 };
 gs_status launch_stencil_f64(gs_ctx* c, const StencilArgs& a);
 // fills the fixed-point fields for plan p and an n-site input held at (m, e)

@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 
 import lattice_inputs as li
+from oracle import dirac
 from tests.gpu_util import lib, to_dev, torch_cuda
 
 pytestmark = pytest.mark.gpu
@@ -23,12 +24,17 @@ def _ctx(gs, torch, dims, m0, U):
 
 
 def _both(env, dims, m0, U, x):
-    """D x by the context and by the double-precision kernel, complex128 [V][12]."""
+    """D x by the context and by the double-precision kernel, or above that one's 8192
+    sites by the oracle's matrix; complex128 [V][12]."""
     torch, gs = env
     ctx = _ctx(gs, torch, dims, m0, U)
     xd = to_dev(x, torch)
     y, ref = torch.empty_like(xd), torch.empty_like(xd)
     ctx.wilson_apply(xd, y)
+    if li.volume(dims) > 8192:
+        torch.cuda.synchronize()
+        ctx.close()
+        return y.cpu().numpy().reshape(-1, 12), (dirac.wilson_matrix(U, dims, m0) @ x.ravel()).reshape(-1, 12)
     assert gs.wilson_apply_noalloc(dims, m0, to_dev(U, torch), xd, ref,
                                    torch.cuda.current_stream().cuda_stream) == gs.GS_OK
     torch.cuda.synchronize()
@@ -126,3 +132,42 @@ def test_applications_back_to_back(env, dims):
     torch.cuda.synchronize()
     assert all(torch.equal(y, alone[k % 3]) for k, y in enumerate(ys))
     ctx.close()
+
+
+def _terms(U, dims, m0, x):
+    """Sum of the moduli of the terms of each component of D x: hops of moduli of links and spinors."""
+    shape = tuple(reversed(dims))
+    A = np.abs(U).reshape(*shape, 4, 3, 3)
+    v = np.abs(x).reshape(*shape, 4, 3)
+    out = abs(m0 + 4) * v
+    for mu in range(4):
+        ax, g = 3 - mu, (3, 2, 1, 0) if mu < 2 else (2, 3, 0, 1)    # |gamma_mu| exchanges these spins
+        h = v + v[..., g, :]
+        out += 0.5 * np.einsum("...ab,...sb->...sa", A[..., mu, :, :], np.roll(h, -1, ax))
+        out += 0.5 * np.roll(np.einsum("...ba,...sb->...sa", A[..., mu, :, :], h), 1, ax)
+    return out.reshape(-1, 12)
+
+
+# Either kernel is off by a few units of the terms' moduli: double precision by at most 61 x 2^-53; fixed
+# point, where a hop contributes at least 2^-8 of the scale, by 21 units of 2^-57 of it (per hop: six dropped
+# products of a quarter unit, two roundings of half a unit, 0.15 for the input): together below 2^-44.
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (4, 6, 5, 8), (8, 10, 8, 24)])
+@pytest.mark.parametrize("links", ["rough", "near the identity", "identity"])
+@pytest.mark.parametrize("uneven", ["spin", "colour", "spin and colour", "one spin only", "sites", "mild"])
+def test_weak_components_keep_their_digits(env, dims, links, uneven):
+    rng = np.random.default_rng(16)
+    V = li.volume(dims)
+    U = li.random_gauge(dims, {"rough": 0.4, "near the identity": 1e-7, "identity": 0.0}[links], 17)
+    x = rng.standard_normal((V, 4, 3)) + 1j * rng.standard_normal((V, 4, 3))
+    if "spin" in uneven:
+        x *= np.array([1.0, 1e-6, 1e-12, 1e-25]).reshape(4, 1)
+    if "colour" in uneven:
+        x *= np.array([1e-9, 1.0, 1e-30])
+    if uneven == "one spin only":
+        x[:, 1:] = 0.0
+    if uneven == "sites":
+        x *= 10.0 ** rng.uniform(-12, 3, (V, 1, 1))
+    if uneven == "mild":
+        x *= np.array([1.0, 2.0 ** -7, 2.0 ** -9, 2.0 ** -14]).reshape(4, 1)
+    y, ref = _both(env, dims, -0.35, U, x.reshape(V, 12))
+    assert np.all(np.abs(y - ref) <= 2.0 ** -44 * _terms(U, dims, -0.35, x))
