@@ -199,7 +199,7 @@ void gs_default_opts(gs_solve_opts* opts);
  * own terms (typically 2^-52), also where those are small beside the other
  * components.  The other FP64 entry points, whose results count by their norms
  * (solves, S_bb, its approximations, residuals), resolve a stencil's result to
- * about 2^-56 of the largest input component around the site. */
+ * 2^-51 (typically 2^-55) of the largest input component around the site. */
 gs_status wilson_apply(gs_ctx* ctx, const void* x_dev, void* y_dev);
 
 /* Site permutation of Section 2 ("Permutation_block": P(p) exchanges the

@@ -77,7 +77,7 @@ struct FxSmem {
     double blk[8];
     double sum[8];
     double2 sc[5];                 // alpha, omega, beta, rho, <rhat, v>
-    int flag, shift;               // shift: exponent that beta's factor in sc[2] leaves out
+    int flag, far;                 // far: beta_far
     double2 vec[RES ? 7 : 1][RES ? 12 : 1][kSitesPerBlock];      // r, rhat, v, t, x, p, s
     int4 link[RES ? 8 : 1][RES ? 9 : 1][kSitesPerBlock];         // [hop][entry][site]
 };
@@ -337,28 +337,28 @@ __device__ __forceinline__ double shift2(double d, int k) {
 }
 __device__ __forceinline__ double2 shift2(double2 v, int k) { return make_double2(shift2(v.x, k), shift2(v.y, k)); }
 
-// beta's factor tt / (rv ts) and, from it, beta = rho' (tt / (rv ts)).  The
-// products grow with the eighth power of the right-hand side's norm, so away
-// from the middle of the range every number goes in with its exponent taken out,
-// and the sum of the exponents k comes back at the end: ||b|| = 1e40 made beta
-// 0 and 1e-40 infinite.  Powers of two change no rounding.
-__device__ __forceinline__ double2 beta_factor(double2 rv, double2 ts, double tt, int& k) {
-    const int er = max_exponent(rv), es = max_exponent(ts), et = fx_exponent((unsigned)__double2hiint(tt));
-    constexpr int mid = 1023, near = 240;
-    k = 0;
-    if (max(max(abs(er - mid), abs(es - mid)), abs(et - mid)) > near) {
-        k = et - er - es + mid;
-        rv = shift2(rv, mid - er);
-        ts = shift2(ts, mid - es);
-        tt = shift2(tt, mid - et);
-    }
-    return zdiv(make_double2(tt, 0.0), zmul(rv, ts));
+// beta = rho' tt / (rv ts).  The products grow with the eighth power of the right-hand
+// side's norm: ||b|| = 1e40 made beta 0 and 1e-40 infinite.  Away from the middle of
+// the range (beta_far) every number therefore goes in with its exponent taken out
+// and the sum of the exponents comes back at the end.  Powers of two change no rounding.
+__device__ __forceinline__ double2 beta_factor(double2 rv, double2 ts, double tt) {      // tt / (rv ts)
+    const double x = fma(rv.x, ts.x, -(rv.y * ts.y)), y = fma(rv.x, ts.y, rv.y * ts.x);
+    const double inv = 1.0 / fma(x, x, y * y);
+    return make_double2(tt * x * inv, -(tt * y) * inv);
 }
-__device__ __forceinline__ double2 beta_of(double2 rho, double2 factor, int k) {
-    const int e = k ? max_exponent(rho) - 1023 : 0;
-    if (e) rho = shift2(rho, -e);
-    const double2 be = zmul(rho, factor);      // one product for both: the same rounding
-    return k ? shift2(be, k + e) : be;
+__device__ __forceinline__ double2 beta_product(double2 a, double2 b) {
+    return make_double2(fma(a.x, b.x, -(a.y * b.y)), fma(a.x, b.y, a.y * b.x));
+}
+__device__ __forceinline__ bool beta_far(double2 rv, double2 ts, double tt) {
+    constexpr int mid = 1023, near = 240;
+    const int et = fx_exponent((unsigned)__double2hiint(tt));
+    return max(max(abs(max_exponent(rv) - mid), abs(max_exponent(ts) - mid)), abs(et - mid)) > near;
+}
+__device__ __noinline__ double2 beta_far_out(double2 rho, double2 rv, double2 ts, double tt) {
+    const int er = max_exponent(rv) - 1023, es = max_exponent(ts) - 1023, e = max_exponent(rho) - 1023;
+    const int et = fx_exponent((unsigned)__double2hiint(tt)) - 1023;
+    return shift2(beta_product(shift2(rho, -e), beta_factor(shift2(rv, -er), shift2(ts, -es), shift2(tt, -et))),
+                  e + et - er - es);
 }
 
 struct FxClock {   // phase clock of block 0 (profiling only)
@@ -539,7 +539,7 @@ __global__ void __launch_bounds__(kT<NS>, NS) k_bicg_persistent_fx(const __grid_
                 break;
             }
             // Serial FP64 algebra: a step takes 0.05 us, so two warps on two
-            // quarters of the SM share it.  beta = (rho' / rho) (alpha / omega)
+            // quarters of the SM share it (and a third looks at the range).  beta = (rho' / rho) (alpha / omega)
             // = rho' <t, t> / (<rhat, v> <t, s>).
             if (threadIdx.x == 0) {
                 const double inv = tot[2] > 0.0 ? 1.0 / tot[2] : 0.0;
@@ -548,14 +548,17 @@ __global__ void __launch_bounds__(kT<NS>, NS) k_bicg_persistent_fx(const __grid_
                 sm.sc[3] = make_double2(tot[6] - (om.x * tot[3] - om.y * tot[4]),
                                         tot[7] - (om.x * tot[4] + om.y * tot[3]));
             } else if (threadIdx.x == 32) {
-                sm.sc[2] = beta_factor(sm.sc[4], make_double2(tot[0], tot[1]), tot[2], sm.shift);
+                sm.sc[2] = beta_factor(sm.sc[4], make_double2(tot[0], tot[1]), tot[2]);
+            } else if (threadIdx.x == 64) {
+                sm.far = beta_far(sm.sc[4], make_double2(tot[0], tot[1]), tot[2]);
             }
             __syncthreads();
             if (threadIdx.x == 0) {
                 const double2 om = sm.sc[1], rho_new = sm.sc[3];
                 int f = (isfinite(om.x) && isfinite(om.y)) ? 0 : 10 + GS_NONFINITE;
                 if (f == 0 && !(om.x == 0.0 && om.y == 0.0) && !(rho_new.x == 0.0 && rho_new.y == 0.0)) {
-                    const double2 be = beta_of(rho_new, sm.sc[2], sm.shift);
+                    const double2 be = sm.far ? beta_far_out(rho_new, sm.sc[4], make_double2(tot[0], tot[1]), tot[2])
+                                              : beta_product(rho_new, sm.sc[2]);
                     sm.sc[2] = be;
                     if (!isfinite(be.x) || !isfinite(be.y)) f = 10 + GS_NONFINITE;
                 } else if (f == 0) {
