@@ -40,8 +40,8 @@ struct gs_net {
     int64_t nel[3] = {};     // complex entries per layer
     long long step = 0;
     // scratch sized for a lattice
-    int64_t capV = 0;
-    int capB = 0;            // samples the activations hold
+    int64_t capV = 0;        // sites of U32
+    int64_t capA = 0;        // sites x samples that the activations hold
     float2* act[4] = {};     // act0 [V][4][3], act1/2 [V][4C][3], act3 [V][4][3]
     float2* gact[2] = {};    // gradient buffers [V][4C][3]
     float2* partial = nullptr;  // [chunks][9][K][R]
@@ -917,31 +917,36 @@ static void gradw_dispatch(int C, int cin, int cout, const float2* in, const flo
     }
 }
 
-// scratch of a network for a lattice of V sites; FP32 links of the context
+// scratch of a network for B samples of a lattice of V sites, which only grows (a
+// network may serve several lattices in turn); FP32 links of the context
 static gs_status net_prepare(gs_ctx* c, gs_net* nt, int B = 1) {
     const int64_t V = c->V;
-    if (nt->capV < V || nt->capB < B) {
-        auto drop = [](auto& a) {
-            cudaFree(a);
-            a = nullptr;       // an allocation below may fail: nothing is freed twice
-        };
+    auto drop = [](auto& a) {
+        cudaFree(a);
+        a = nullptr;       // an allocation below may fail: nothing is freed twice
+    };
+    auto failed = [&]() {
+        cudaGetLastError();
+        return set_err(c, GS_ENOMEM, "allocating network activations failed");
+    };
+    if (nt->capA < B * V) {
         for (auto& a : nt->act) drop(a);
         for (auto& a : nt->gact) drop(a);
-        drop(nt->U32);
-        nt->U32_src = nullptr;
+        nt->capA = 0;
         const size_t big = (size_t)B * V * 4 * nt->C * 3 * sizeof(float2);
         const size_t sm = (size_t)B * V * 12 * sizeof(float2);
         if (cudaMalloc(&nt->act[0], sm) != cudaSuccess || cudaMalloc(&nt->act[1], big) != cudaSuccess ||
             cudaMalloc(&nt->act[2], big) != cudaSuccess || cudaMalloc(&nt->act[3], sm) != cudaSuccess ||
-            cudaMalloc(&nt->gact[0], big) != cudaSuccess || cudaMalloc(&nt->gact[1], big) != cudaSuccess ||
-            cudaMalloc(&nt->U32, (size_t)V * 36 * sizeof(float2)) != cudaSuccess) {
-            cudaGetLastError();
-            nt->capV = 0;
-            nt->capB = 0;
-            return set_err(c, GS_ENOMEM, "allocating network activations failed");
-        }
+            cudaMalloc(&nt->gact[0], big) != cudaSuccess || cudaMalloc(&nt->gact[1], big) != cudaSuccess)
+            return failed();
+        nt->capA = B * V;
+    }
+    if (nt->capV < V) {
+        drop(nt->U32);
+        nt->U32_src = nullptr;
+        nt->capV = 0;
+        if (cudaMalloc(&nt->U32, (size_t)V * 36 * sizeof(float2)) != cudaSuccess) return failed();
         nt->capV = V;
-        nt->capB = B;
     }
     if (nt->U32_src != (const void*)c || !c->net_links_fresh) {
         k_links32<<<grid_for(V * 36, 256, c->num_sms * 8), 256, 0, c->stream>>>(c->U_abi, nt->U32, V * 36);

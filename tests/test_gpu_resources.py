@@ -1,0 +1,55 @@
+"""What calls hold and share between them: a network's buffers on several
+lattices, memory, the blocks of batched solves, and the routes of fields that
+fixed point cannot hold."""
+import numpy as np
+import pytest
+
+import lattice_inputs as li
+from oracle import net as onet
+from tests.gpu_util import lib, to_dev, torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = torch_cuda()
+    return torch, lib()
+
+
+def _ctx(gs, torch, dims, m0, U, stream=None):
+    ctx = gs.Context(dims, m0, torch.cuda.current_stream().cuda_stream if stream is None else stream)
+    ctx.set_gauge(to_dev(U, torch))
+    return ctx
+
+
+def _net(gs, seed):
+    nt = gs.Net(24)
+    for l, w in enumerate(onet.init_weights(24, seed, scale=0.25)):
+        nt.set_weights(l, w.astype(np.complex64))
+    return nt
+
+
+def test_network_on_two_lattices_keeps_its_buffers(env):
+    """Training in groups of samples on a small lattice and applying on a large one in
+    turn: nothing is allocated or freed once both have been seen."""
+    torch, gs = env
+    small, large = (4, 4, 4, 4), (8, 8, 8, 32)
+    cs, cl = (_ctx(gs, torch, d, 0.1, li.random_gauge(d, 0.3, 1)) for d in (small, large))
+    rng = np.random.default_rng(2)
+    t, z = (to_dev((rng.standard_normal((4, 240, 12)) + 1j * rng.standard_normal((4, 240, 12))).astype(np.complex64),
+                   torch) for _ in range(2))
+    x = to_dev(rng.standard_normal((8192, 12)) + 0j, torch)
+    ys = [torch.empty_like(x) for _ in range(2)]
+    nt = _net(gs, 3)
+    losses, free = [], []
+    for k in range(2):
+        losses.append(nt.train_step(cs.handle, 1, 0, 0, 4, t, z, 0.0, update=False))
+        free.append(torch.cuda.mem_get_info()[0])
+        nt.apply(cl.handle, 2, 0, 0, x, ys[k])
+        free.append(torch.cuda.mem_get_info()[0])
+    assert free[1] == free[2] == free[3]
+    assert losses[0] == losses[1] and torch.equal(ys[0], ys[1])
+    nt.close()
+    cs.close()
+    cl.close()
