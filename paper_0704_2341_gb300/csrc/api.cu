@@ -2,6 +2,8 @@
 // wilson_apply, permute_sites, schur_apply and schur_solve.
 #include <math.h>
 
+#include <atomic>
+
 #include "fx.cuh"
 
 using namespace gs;
@@ -295,7 +297,8 @@ gs_status gs_set_gauge(gs_ctx* c, const void* U_dev) {
                                cudaMemcpyDeviceToDevice, c->stream));
     c->have_gauge = true;
     c->gauge_gen++;
-    c->net_links_fresh = false;
+    static std::atomic<unsigned long long> fields{0};
+    c->field_id = ++fields;
     invalidate_mixed_links(c);
     for (Plan* p : c->plans) {
         gs_status s = pack_plan_links(c, p);

@@ -262,7 +262,7 @@ struct gs_ctx {
     unsigned gauge_gen = 0;            // counts gs_set_gauge calls
     unsigned lane_gauge_gen = 0;       // (lane contexts) the parent's gauge_gen their field was copied at
     struct gs_net* net = nullptr;      // learned preconditioner attached with gs_set_net (net.cu)
-    bool net_links_fresh = false;      // the network's FP32 link copy matches U_abi
+    unsigned long long field_id = 0;   // names the field: another one for every gs_set_gauge of the process
     float2 *fg_V = nullptr, *fg_Z = nullptr, *fg_w = nullptr;  // FGMRES-net vectors (FP32 stencil layout)
     int64_t fg_cap = 0;
     int fg_m = 0;

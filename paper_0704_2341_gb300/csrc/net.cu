@@ -45,8 +45,8 @@ struct gs_net {
     float2* act[4] = {};     // act0 [V][4][3], act1/2 [V][4C][3], act3 [V][4][3]
     float2* gact[2] = {};    // gradient buffers [V][4C][3]
     float2* partial = nullptr;  // [chunks][9][K][R]
-    float2* U32 = nullptr;      // FP32 links [V][4][9] (site order) of the last context
-    const void* U32_src = nullptr;
+    float2* U32 = nullptr;      // FP32 links [V][4][9] (site order)
+    unsigned long long U32_field = 0;   // the field (gs_ctx::field_id) they are the links of
     float* red = nullptr;       // small reduction scratch
     unsigned int* counter = nullptr;
     float* host_red = nullptr;
@@ -943,17 +943,16 @@ static gs_status net_prepare(gs_ctx* c, gs_net* nt, int B = 1) {
     }
     if (nt->capV < V) {
         drop(nt->U32);
-        nt->U32_src = nullptr;
+        nt->U32_field = 0;
         nt->capV = 0;
         if (cudaMalloc(&nt->U32, (size_t)V * 36 * sizeof(float2)) != cudaSuccess) return failed();
         nt->capV = V;
     }
-    if (nt->U32_src != (const void*)c || !c->net_links_fresh) {
+    if (nt->U32_field != c->field_id) {
         k_links32<<<grid_for(V * 36, 256, c->num_sms * 8), 256, 0, c->stream>>>(c->U_abi, nt->U32, V * 36);
         c->launches++;
         GS_CHECK_LAUNCH(c);
-        nt->U32_src = c;
-        c->net_links_fresh = true;
+        nt->U32_field = c->field_id;
     }
     return GS_OK;
 }

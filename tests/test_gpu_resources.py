@@ -53,3 +53,28 @@ def test_network_on_two_lattices_keeps_its_buffers(env):
     nt.close()
     cs.close()
     cl.close()
+
+
+def test_two_networks_follow_a_new_field(env):
+    """Each network of a context copies the new field's links, whichever is used first."""
+    torch, gs = env
+    dims = (4, 4, 4, 4)
+    U1, U2 = li.random_gauge(dims, 0.3, 4), li.random_gauge(dims, 0.4, 5)
+    x = to_dev(np.random.default_rng(6).standard_normal((128, 12)) + 0j, torch)
+
+    def apply(ctx, nt):
+        y = torch.empty_like(x)
+        nt.apply(ctx.handle, 2, 0, 0, x, y)
+        return y
+
+    ctx, fresh = _ctx(gs, torch, dims, 0.1, U1), _ctx(gs, torch, dims, 0.1, U2)
+    a, b, c = _net(gs, 7), _net(gs, 7), _net(gs, 7)
+    apply(ctx, a)
+    apply(ctx, b)
+    ctx.set_gauge(to_dev(U2, torch))
+    want = apply(fresh, c)
+    assert torch.equal(apply(ctx, a), want) and torch.equal(apply(ctx, b), want)
+    for n in (a, b, c):
+        n.close()
+    ctx.close()
+    fresh.close()
