@@ -899,7 +899,7 @@ static void conv_dispatch(int C, int cin, int cout, const float2* in, float2* ou
         case 2: conv_dispatch_t<2, WT>(cin, cout, in, out, W, U32, nbr, V, blocks, s); break;
         case 4: conv_dispatch_t<4, WT>(cin, cout, in, out, W, U32, nbr, V, blocks, s); break;
         case 8: conv_dispatch_t<8, WT>(cin, cout, in, out, W, U32, nbr, V, blocks, s); break;
-        default:   // 24 channels in FP32: train_group
+        default:   // 24 channels; in FP32 net_forward refuses them
             if constexpr (std::is_same<WT, __nv_bfloat162>::value)
                 conv_dispatch_t<24, WT>(cin, cout, in, out, W, U32, nbr, V, blocks, s);
             break;
@@ -913,7 +913,7 @@ static void gradw_dispatch(int C, int cin, int cout, const float2* in, const flo
         case 2: gradw_dispatch_t<2>(cin, cout, in, gout, partial, U32, nbr, V, s); break;
         case 4: gradw_dispatch_t<4>(cin, cout, in, gout, partial, U32, nbr, V, s); break;
         case 8: gradw_dispatch_t<8>(cin, cout, in, gout, partial, U32, nbr, V, s); break;
-        default: break;   // 24 channels: train_group
+        default: break;   // 24 channels never get here (net_forward)
     }
 }
 
@@ -962,6 +962,8 @@ static gs_status net_forward(gs_ctx* c, gs_net* nt, bool bf16) {
     const Plan* id = c->plans[0];
     const int64_t V = c->V;
     const int blocks = (int)((V + kTS - 1) / kTS);
+    // the FP32 kernels of that width work on groups of samples (train_group)
+    if (!bf16 && nt->C == kC) return set_err(c, GS_EINVAL, "24 channels in FP32: train_group, not net_forward");
     for (int l = 0; l < 3; ++l) {
         int cin, cout;
         layer_dims(nt->C, l, &cin, &cout);
