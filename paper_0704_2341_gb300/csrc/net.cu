@@ -328,7 +328,10 @@ __device__ __forceinline__ void load6(const float2* p, float2 (&v)[6]) {
     }
 }
 
-// partial[chunk][d][k][R] of the C -> C layer: grid (chunks of a sample, 9, samples)
+// partial[chunk][d][k][R] of the C -> C layer: grid (chunks of a sample, 9, samples).
+// A chain of FP32 sums runs over 1 / kChunks of a sample's sites; a block of a
+// group of samples takes several such parts and adds them in memory (its own 74
+// KB, in L2), so that sharing a launch makes no chain longer.
 __global__ void __launch_bounds__(256, 2) k_net_gradw24(const float2* __restrict__ in, const float2* __restrict__ gout,
                                                        float2* __restrict__ partial, const float2* __restrict__ U32,
                                                        const int2* __restrict__ nbr, int64_t V) {
@@ -338,10 +341,34 @@ __global__ void __launch_bounds__(256, 2) k_net_gradw24(const float2* __restrict
     in += (int64_t)blockIdx.z * V * kRows * 3;
     gout += (int64_t)blockIdx.z * V * kRows * 3;
     const int64_t tiles = (V + kTS - 1) / kTS;
-    const int64_t t0 = tiles * blockIdx.x / gridDim.x, t1 = tiles * (blockIdx.x + 1) / gridDim.x;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;     // rows R = 6 tx .., k = 6 ty ..
+    const int q0 = kChunks * blockIdx.x / gridDim.x, q1 = kChunks * (blockIdx.x + 1) / gridDim.x;
+    const int64_t t0 = tiles * q0 / kChunks, t1 = tiles * q1 / kChunks;
+    float4* const dst = (float4*)(partial + (chunk * 9 + d) * (kRows * kRows) + 6 * ty * kRows + 6 * tx);
     float2 c[6][6] = {};
+    int64_t part = t0 + (tiles + kChunks - 1) / kChunks;        // the tile at which the part ends
+    bool first = true;
+    auto flush = [&]() {
+#pragma unroll
+        for (int i = 0; i < 6; ++i)
+#pragma unroll
+            for (int j = 0; j < 6; j += 2) {
+                float4* const o = dst + (i * kRows + j) / 2;
+                float4 v = first ? make_float4(0.f, 0.f, 0.f, 0.f) : *o;
+                v.x += c[i][j].x;
+                v.y += c[i][j].y;
+                v.z += c[i][j + 1].x;
+                v.w += c[i][j + 1].y;
+                *o = v;
+                c[i][j] = c[i][j + 1] = make_float2(0.f, 0.f);
+            }
+        first = false;
+    };
     for (int64_t tile = t0; tile < t1; ++tile) {
+        if (tile == part) {
+            flush();
+            part += (tiles + kChunks - 1) / kChunks;
+        }
         const int64_t base = tile * kTS;
         for (int e = threadIdx.x; e < kTS * kRows; e += 256) {
             const int s = e / kRows, k = e - s * kRows;
@@ -367,11 +394,7 @@ __global__ void __launch_bounds__(256, 2) k_net_gradw24(const float2* __restrict
         }
         __syncthreads();
     }
-    float2* dst = partial + (chunk * 9 + d) * (kRows * kRows);
-#pragma unroll
-    for (int i = 0; i < 6; ++i)
-#pragma unroll
-        for (int j = 0; j < 6; ++j) dst[(6 * ty + i) * kRows + 6 * tx + j] = c[i][j];
+    flush();
 }
 
 // out = sum_d W_d T_d of the C -> C layer: tiles of 16 sites (48 columns) by all
