@@ -117,6 +117,9 @@ struct Plan {
     double2* links = nullptr;    // [V][4][9] -1/2 U_mu(perm[j]) in label order
     int4* fx_links = nullptr;    // the same in fixed point (fx.cuh): limbs (re.lo, re.hi, im.lo, im.hi)
     int* fx_flag = nullptr;      // device: 1 if a link lies outside fixed point's range
+    volatile unsigned* fit_host = nullptr;   // the same for the host, in mapped memory: 2 fit_gen + fx_flag once the
+    unsigned* fit_dev = nullptr;             // links of generation fit_gen are packed
+    unsigned fit_gen = 0;
     bool links_ready = false;
     long long hops[2][2] = {{0, 0}, {0, 0}};  // [out set][in set] in-set neighbour terms (0 = b, 1 = r)
     double2* dtinv = nullptr;    // [V - nb][12][12] inverse block row sums of D_rr (Reusken), lazily
@@ -359,6 +362,11 @@ struct StencilArgs {
                              // the other callers' vectors matter by their norms
 };
 gs_status launch_stencil_f64(gs_ctx* c, const StencilArgs& a);
+// whether fixed point holds plan p's links: 1, 0, or -1 if the host does not know yet
+inline int plan_fits(const Plan* p) {
+    const unsigned w = *p->fit_host;
+    return (w >> 1) != (p->fit_gen & 0x7fffffffu) ? -1 : !(w & 1u);
+}
 // fills the fixed-point fields for plan p and an n-site input held at (m, e)
 void fx_args(const Plan* p, const longlong2* m, const int* e, int64_t n, StencilArgs* a);
 gs_status launch_stencil_fx(gs_ctx* c, const StencilArgs& a, int grid);

@@ -165,6 +165,11 @@ __global__ void __launch_bounds__(256) k_pack_links(int64_t V, const int32_t* __
     }
 }
 
+// The packed links' flag for the host (Plan::fit_host).
+__global__ void k_publish_fit(const int* __restrict__ flag, unsigned gen, unsigned* host) {
+    *(volatile unsigned*)host = 2u * gen + (*flag != 0 ? 1u : 0u);
+}
+
 // y[i] = x[perm[i]] per site (12 complex), and the transpose.
 __global__ void k_gather(const int32_t* __restrict__ perm, const double2* __restrict__ x,
                          double2* __restrict__ y, int64_t nsites) {
@@ -203,6 +208,7 @@ void free_plan(Plan* p) {
     cudaFree(p->links);
     cudaFree(p->fx_links);
     cudaFree(p->fx_flag);
+    if (p->fit_host) cudaFreeHost((void*)p->fit_host);
     cudaFree(p->dtinv);
     delete p;
 }
@@ -212,7 +218,8 @@ gs_status pack_plan_links(gs_ctx* c, Plan* p) {
     GS_CUDA(c, cudaMemsetAsync(p->fx_flag, 0, sizeof(int), c->stream));
     k_pack_links<<<grid_for(c->V, 32, c->num_sms * 16), 256, 0, c->stream>>>(c->V, p->perm, c->U_abi, p->links,
                                                                             p->fx_links, p->fx_flag);
-    c->launches++;
+    k_publish_fit<<<1, 1, 0, c->stream>>>(p->fx_flag, ++p->fit_gen, p->fit_dev);
+    c->launches += 2;
     GS_CHECK_LAUNCH(c);
     p->links_ready = true;
     p->dtinv_ready = false;   // the Reusken block inverses depend on the links
@@ -252,12 +259,15 @@ gs_status get_plan(gs_ctx* c, int type, int dir, int inverse, Plan** out) {
         cudaMalloc(&p->nbr, V * 4 * sizeof(int2)) != cudaSuccess ||
         cudaMalloc(&p->links, V * 36 * sizeof(double2)) != cudaSuccess ||
         cudaMalloc(&p->fx_links, fx_padded(V) * 36 * sizeof(int4)) != cudaSuccess ||
-        cudaMalloc(&p->fx_flag, sizeof(int)) != cudaSuccess) {
+        cudaMalloc(&p->fx_flag, sizeof(int)) != cudaSuccess ||
+        cudaHostAlloc((void**)&p->fit_host, sizeof(unsigned), cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostGetDevicePointer((void**)&p->fit_dev, (void*)p->fit_host, 0) != cudaSuccess) {
         free_plan(p);
         cudaGetLastError();
         return set_err(c, GS_ENOMEM, "allocating a permutation plan for V = %lld failed",
                        (long long)V);
     }
+    *p->fit_host = 0;
     Dims d;
     for (int mu = 0; mu < 4; ++mu) d.L[mu] = c->dims[mu];
     const int g = grid_for(V, 256, c->num_sms * 8);

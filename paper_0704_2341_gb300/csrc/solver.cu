@@ -152,9 +152,12 @@ gs_status inner_solve_f64(gs_ctx* c, const Plan* p, const double2* t, double2* z
 
     volatile BicgPublic* pub = w.pub_host;
     int kernel = c->opt_inner_kernel;
+    if (plan_fits(p) < 0) GS_CUDA(c, cudaStreamSynchronize(c->stream));   // so that the choice does not depend on timing
+    const bool fits = plan_fits(p) != 0;
+    if (kernel == 0 && !fits && c->ledger) kernel = 1;
     if (kernel == 0) {
-        // the whole solve in one cooperative launch (persistent_fx.cu); a field
-        // or right-hand side that fixed point cannot hold goes to the
+        // the whole solve in one cooperative launch (persistent_fx.cu); a field (known
+        // beforehand) or right-hand side that fixed point cannot hold goes to the
         // double-precision kernel (persistent.cu), or inside a batched call,
         // whose block ledger counts blocks of one size, to the per-phase launches.
         // So does a solve that ended on a zero inner product: the integer sums
@@ -168,10 +171,12 @@ gs_status inner_solve_f64(gs_ctx* c, const Plan* p, const double2* t, double2* z
             GS_CUDA(c, cudaEventSynchronize(w.ev[0]));
             return GS_OK;
         };
-        s = persistent_bicg_fx(c, p, k1, t, z, w, o.inner_tol, o.inner_max_iter);
-        if (s != GS_OK || (s = finished()) != GS_OK) return s;
-        ledger_release(c);
-        if (pub->status == kFxUnfit || pub->status == GS_BREAKDOWN) {
+        if (fits) {
+            s = persistent_bicg_fx(c, p, k1, t, z, w, o.inner_tol, o.inner_max_iter);
+            if (s != GS_OK || (s = finished()) != GS_OK) return s;
+            ledger_release(c);
+        }
+        if (!fits || pub->status == kFxUnfit || pub->status == GS_BREAKDOWN) {
             if (c->ledger) kernel = 1;
             else {
                 s = persistent_bicg_f64(c, k1, k3, t, z, w, n, o.inner_tol, o.inner_max_iter);

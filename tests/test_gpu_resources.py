@@ -78,3 +78,36 @@ def test_two_networks_follow_a_new_field(env):
         n.close()
     ctx.close()
     fresh.close()
+
+
+@pytest.mark.parametrize("inner", [0, 1])
+def test_field_beyond_fixed_point_goes_straight_to_double_precision(env, inner):
+    """One link far from unitary: no conversion, no attempt of the fixed-point solver.
+    S_bb x = two stencils and an inner solve, as kernels: 3 in one cooperative launch,
+    and with one launch per phase the two stencils an iteration are single ones."""
+    torch, gs = env
+    dims, V = (4, 6, 4, 8), 768
+    U = li.random_gauge(dims, 0.3, 8)
+    bad = U.copy()
+    bad[V // 2, 1, 0, 2] = 1.5            # an entry above 1.01
+    rng = np.random.default_rng(9)
+    x = to_dev(rng.standard_normal((V // 16, 12)) + 1j * rng.standard_normal((V // 16, 12)), torch)
+    y, ref = torch.empty_like(x), torch.empty_like(x)
+    o = gs.gs_default_opts(inner_tol=1e-12)
+    ctx = _ctx(gs, torch, dims, 0.1, bad)
+    ctx.set_option(gs.GS_OPT_INNER_KERNEL, inner)
+    ctx.schur_apply(1, 0, 0, x, y, o)
+    st = ctx.schur_apply(1, 0, 0, x, y, o)
+    if inner == 0:
+        assert st.kernel_launches == 3
+    else:      # init, then five launches an iteration, at most two iterations queued past the last
+        assert st.kernel_launches <= 3 + 5 * (st.inner_iters + 2)
+    # the fixed-point route of a field within its range, a rounding away from the same operator
+    good = bad.copy()
+    good[V // 2, 1] *= 0.5
+    ctx.set_gauge(to_dev(good, torch))
+    ctx.schur_apply(1, 0, 0, x, ref, o)
+    ctx.set_gauge(to_dev(bad, torch))
+    ctx.schur_apply(1, 0, 0, x, ref, o)
+    assert torch.equal(y, ref)
+    ctx.close()
