@@ -219,6 +219,10 @@ void ledger_leave(BlockLedger* L, const gs_ctx* c);
 // target, at least `least`, never more than the others leave free; 0 if they
 // did not become free within the context's wait limit x 60
 int64_t ledger_grant(gs_ctx* c, int64_t capacity, int64_t want, int64_t target, int64_t least = 1);
+// The blocks of one FP64 batched call: those of the fixed-point solver that are
+// co-resident at per_sm an SM, less some slots for the other solves' small kernels.
+inline int64_t ledger_capacity(int per_sm, int num_sms) { return (int64_t)per_sm * num_sms - num_sms / 4; }
+constexpr int kFxBatchPerSm = 2;
 // c's last grid has ended (the host has waited for it): its blocks are free
 void ledger_release(gs_ctx* c);
 }  // namespace gs

@@ -656,15 +656,14 @@ __global__ void __launch_bounds__(kPThreads) k_selftest_grid_timeout(GridSync g,
 
 // co-resident grid for a cooperative launch on a set of rest_sites sites: at
 // most `want` blocks.  Inside schur_solve_batched (no GS_OPT_COOP_BLOCKS) the
-// grid comes from the call's block ledger (only the low-precision solver gets here
-// with one: the FP64 solver of a batched call is persistent_fx.cu's): on a small
-// rest set a kernel that passes `round` (the blocks for one pass over the set)
-// asks for exactly that -- FP32 inner solves on 8^4, 96 sites per block, 84.9
-// solves/s against 75.8 with 76 blocks each; otherwise it asks for its share
-// of the GPU while n solves run (two blocks per SM on small sets, all
-// co-resident blocks on large ones).
+// grid comes from the call's block ledger: on a small rest set the blocks for one
+// pass over the set, `round` -- FP32 inner solves on 8^4, 96 sites per block, 84.9
+// solves/s against 75.8 with 76 blocks each; on others its share of the GPU while
+// n solves run (two blocks per SM on small sets, all co-resident blocks on
+// large ones).  `capacity`: what the ledger hands out in all, if its blocks are not
+// this kernel's own.
 template <class K>
-static int coop_grid(gs_ctx* c, K kernel, int64_t want, int64_t rest_sites, int64_t round = 0) {
+static int coop_grid(gs_ctx* c, K kernel, int64_t want, int64_t rest_sites, int64_t round, int64_t capacity = 0) {
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kPThreads, 0) != cudaSuccess ||
         per_sm < 1) {
@@ -680,7 +679,7 @@ static int coop_grid(gs_ctx* c, K kernel, int64_t want, int64_t rest_sites, int6
         const bool small = rest_sites <= kBatchMaxRestSites;
         const int64_t target = (small && round > 0) ? round
                                : (small && per_sm > 2 ? 2 : per_sm) * (int64_t)c->num_sms / n;
-        return (int)ledger_grant(c, full, w, target > 0 ? target : 1);
+        return (int)ledger_grant(c, capacity > 0 ? capacity : full, w, target > 0 ? target : 1);
     }
     int64_t g = coop_blocks(c, per_sm, rest_sites);
     if (want < g) g = want;
@@ -730,7 +729,10 @@ gs_status persistent_bicg_f64(gs_ctx* c, const StencilArgs& A, const StencilArgs
     if (s != GS_OK) return s;
     const int64_t tiles = (A.n_out + kSitesPerBlock - 1) / kSitesPerBlock;
     const int64_t want = tiles > (int64_t)c->num_sms ? tiles : (int64_t)c->num_sms;
-    const int g = coop_grid(c, k_bicg_persistent_f64, want, A.n_out, tiles);
+    // The FP64 ledger counts the fixed-point solver's blocks (256 threads, 128
+    // registers, 41 KB or more); this kernel's (128, 168, 27 KB) fit where one of
+    // those does, so they are counted as such.
+    const int g = coop_grid(c, k_bicg_persistent_f64, want, A.n_out, tiles, ledger_capacity(kFxBatchPerSm, c->num_sms));
     if (g < 1) return set_err(c, GS_ECUDA, "no co-resident grid for the persistent solver");
     // tiles of up to 32 sites, no more than the grid needs to cover the rest set
     // once (3840 sites on 152 blocks: 26 per tile, so every SM shares the work)

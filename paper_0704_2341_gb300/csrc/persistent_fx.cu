@@ -694,8 +694,7 @@ static gs_status launch_fx_solver(gs_ctx* c, PArgsFx& P, const FxScratch* f) {
     if (c->coop_block_cap > 0) {
         if (g > c->coop_block_cap) g = c->coop_block_cap;
     } else if (c->ledger) {
-        // some block slots stay free for the other solves' small kernels
-        const int64_t usable = g - c->num_sms / 4;
+        const int64_t usable = ledger_capacity(per_sm, c->num_sms);
         const int64_t n = c->ledger->running.load() > 1 ? c->ledger->running.load() : 1;
         const int64_t share = RES ? tiles : usable / n;
         g = ledger_grant(c, usable, tiles, share > 0 ? share : 1, RES ? tiles : 1);

@@ -151,18 +151,14 @@ gs_status inner_solve_f64(gs_ctx* c, const Plan* p, const double2* t, double2* z
     k3.red = w.red;
 
     volatile BicgPublic* pub = w.pub_host;
-    int kernel = c->opt_inner_kernel;
     if (plan_fits(p) < 0) GS_CUDA(c, cudaStreamSynchronize(c->stream));   // so that the choice does not depend on timing
-    const bool fits = plan_fits(p) != 0;
-    if (kernel == 0 && !fits && c->ledger) kernel = 1;
-    if (kernel == 0) {
+    if (c->opt_inner_kernel == 0) {
         // the whole solve in one cooperative launch (persistent_fx.cu); a field (known
         // beforehand) or right-hand side that fixed point cannot hold goes to the
-        // double-precision kernel (persistent.cu), or inside a batched call,
-        // whose block ledger counts blocks of one size, to the per-phase launches.
-        // So does a solve that ended on a zero inner product: the integer sums
-        // give an exact zero where the large terms cancel below 2^-54 of the
-        // largest, and only sums in double precision tell that from a breakdown.
+        // double-precision kernel (persistent.cu).  So does a solve that ended on a
+        // zero inner product: the integer sums give an exact zero where the large
+        // terms cancel below 2^-54 of the largest, and only sums in double precision
+        // tell that from a breakdown.
         int slot = -1;
         if (c->prof.on && (s = prof_begin(c, &slot)) != GS_OK) return s;
         auto finished = [&]() -> gs_status {
@@ -171,17 +167,16 @@ gs_status inner_solve_f64(gs_ctx* c, const Plan* p, const double2* t, double2* z
             GS_CUDA(c, cudaEventSynchronize(w.ev[0]));
             return GS_OK;
         };
+        const bool fits = plan_fits(p) != 0;
         if (fits) {
             s = persistent_bicg_fx(c, p, k1, t, z, w, o.inner_tol, o.inner_max_iter);
             if (s != GS_OK || (s = finished()) != GS_OK) return s;
             ledger_release(c);
         }
         if (!fits || pub->status == kFxUnfit || pub->status == GS_BREAKDOWN) {
-            if (c->ledger) kernel = 1;
-            else {
-                s = persistent_bicg_f64(c, k1, k3, t, z, w, n, o.inner_tol, o.inner_max_iter);
-                if (s != GS_OK || (s = finished()) != GS_OK) return s;
-            }
+            s = persistent_bicg_f64(c, k1, k3, t, z, w, n, o.inner_tol, o.inner_max_iter);
+            if (s != GS_OK || (s = finished()) != GS_OK) return s;
+            ledger_release(c);
         }
         if (slot >= 0) {
             // algorithmic FP64 work: two D_rr applications per iteration and the
@@ -197,8 +192,7 @@ gs_status inner_solve_f64(gs_ctx* c, const Plan* p, const double2* t, double2* z
                 {slot, 3, (long long)(2 * it * nr), (long long)(2 * it * hops),
                  it * (2.0 * fl + 84.0 * (double)n), it * (2.0 * by + 14.0 * 16.0 * (double)n)});
         }
-    }
-    if (kernel != 0) {
+    } else {
         if ((s = launch_bicg_init(c, w, t, z, n, o.inner_tol)) != GS_OK) return s;
         // Iterations are queued ahead of the GPU; the host waits on the event of
         // the iteration `depth` behind and reads the mapped `done` flag, so at most

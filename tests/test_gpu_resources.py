@@ -111,3 +111,36 @@ def test_field_beyond_fixed_point_goes_straight_to_double_precision(env, inner):
     ctx.schur_apply(1, 0, 0, x, ref, o)
     assert torch.equal(y, ref)
     ctx.close()
+
+
+@pytest.mark.parametrize("dims,fields", [((8, 8, 8, 12), "within"), ((8, 8, 8, 12), "beyond"), ((4, 4, 4, 8), "beyond"),
+                                         ((8, 8, 8, 8), "both"), ((8, 8, 8, 12), "both")])
+def test_batched_fp64_solves(env, dims, fields):
+    """Six FP64 solves at once: rest sets above 32 sites per SM (5760: the solves share the
+    co-resident blocks, a part of their tiles each) and below, fields within and beyond fixed
+    point's range, and the two solvers' blocks side by side.  Every inner solve stays one
+    cooperative launch and the solutions are those of one solve at a time."""
+    torch, gs = env
+    streams = [torch.cuda.Stream() for _ in range(6)]
+    V, o = li.volume(dims), gs.gs_default_opts()
+    ctxs, probs = [], []
+    for k, s in enumerate(streams):
+        U = li.random_gauge(dims, 0.3, 40 + k)
+        if fields == "beyond" or (fields == "both" and k % 2):
+            U[V // 3, 2, 1, 1] = 1.2
+        ctxs.append(_ctx(gs, torch, dims, 0.0, U, s.cuda_stream))
+        f = to_dev(li.gaussian_source(dims, 50 + k), torch)
+        probs.append(dict(ctx=ctxs[-1].handle, type=1 + k % 2, dir=0, inverse=k // 4, nrhs=1, f=f, x=torch.zeros_like(f)))
+    ctxs[0].set_option(gs.GS_OPT_BATCH_LANES, 6)
+    torch.cuda.synchronize()
+    for _ in range(2):
+        status, stats = gs.schur_solve_batched(probs, o)
+        assert status == gs.GS_OK
+    for c, pr, st in zip(ctxs, probs, stats):
+        x1 = torch.zeros_like(pr["f"])
+        one = c.schur_solve(pr["type"], 0, pr["inverse"], pr["f"], x1, o)
+        assert st.true_residual <= 1e-10 and one.true_residual <= 1e-10
+        assert (pr["x"] - x1).norm() <= 1e-8 * x1.norm()
+        # as many launches as alone, up to an outer iteration or two (19 launches at most)
+        assert st.kernel_launches <= one.kernel_launches + 40
+        c.close()
