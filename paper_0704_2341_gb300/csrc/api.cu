@@ -101,8 +101,6 @@ gs_status gs_create(gs_ctx** out, const int dims[4], double m0, void* stream) {
     }
     const size_t vbytes = (size_t)V * kSiteC * sizeof(double2);
     bool ok = cudaMalloc(&c->U_abi, (size_t)V * 36 * sizeof(double2)) == cudaSuccess &&
-              cudaMalloc(&c->fx_m, (size_t)fx_padded(V) * kSiteC * sizeof(longlong2)) == cudaSuccess &&
-              cudaMalloc(&c->fx_e, (size_t)V * sizeof(int)) == cudaSuccess &&
               cudaMalloc(&c->full_a, vbytes) == cudaSuccess &&
               cudaMalloc(&c->full_b, vbytes) == cudaSuccess &&
               cudaMalloc(&c->full_c, vbytes) == cudaSuccess &&
@@ -125,6 +123,13 @@ gs_status gs_create(gs_ctx** out, const int dims[4], double m0, void* stream) {
     if (s != GS_OK) {
         gs_destroy(c);
         return s;
+    }
+    const size_t fx_bytes = (size_t)fx_padded(V) * kSiteC * sizeof(longlong2);
+    if (!fx_room(fx_bytes) || cudaMalloc(&c->fx_m, fx_bytes) != cudaSuccess ||
+        cudaMalloc(&c->fx_e, (size_t)V * sizeof(int)) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(c->fx_m);
+        c->fx_m = nullptr;
     }
     *out = c;
     return GS_OK;

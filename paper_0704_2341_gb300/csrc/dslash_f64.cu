@@ -58,7 +58,7 @@ gs_status launch_stencil_f64(gs_ctx* c, const StencilArgs& args) {
     const int64_t blocks_needed = (a.n_out + kSitesPerBlock - 1) / kSitesPerBlock;
     int max_blocks = (a.epi == EPI_NONE) ? (1 << 30) : kMaxRedBlocks;
     const int g = (int)(blocks_needed < max_blocks ? blocks_needed : max_blocks);
-    if (plan_fits(a.plan) == 0) {
+    if (!c->fx_m || plan_fits(a.plan) == 0) {
         switch (a.epi) {
             case EPI_NONE: k_dslash_f64<EPI_NONE><<<g, kThreads, 0, c->stream>>>(a); break;
             case EPI_DOT_RHAT_V: k_dslash_f64<EPI_DOT_RHAT_V><<<g, kThreads, 0, c->stream>>>(a); break;

@@ -115,7 +115,7 @@ struct Plan {
     int32_t* label = nullptr;    // [V] site -> label
     int2* nbr = nullptr;         // [V][4] (fwd label, bwd label) per mu, label-indexed
     double2* links = nullptr;    // [V][4][9] -1/2 U_mu(perm[j]) in label order
-    int4* fx_links = nullptr;    // the same in fixed point (fx.cuh): limbs (re.lo, re.hi, im.lo, im.hi)
+    int4* fx_links = nullptr;    // the same in fixed point (fx.cuh): limbs (re.lo, re.hi, im.lo, im.hi); null: no room
     int* fx_flag = nullptr;      // device: 1 if a link lies outside fixed point's range
     volatile unsigned* fit_host = nullptr;   // the same for the host, in mapped memory: 2 fit_gen + fx_flag once the
     unsigned* fit_dev = nullptr;             // links of generation fit_gen are packed
@@ -238,7 +238,7 @@ struct gs_ctx {
     std::vector<gs::Plan*> plans;      // plans[0] = identity
     gs::InnerWork inner;
     gs::OuterWork outer;
-    longlong2* fx_m = nullptr;         // fixed-point copy of a stencil input (fx.cuh): mantissas
+    longlong2* fx_m = nullptr;         // fixed-point copy of a stencil input (fx.cuh): mantissas (null: no room)
     int* fx_e = nullptr;               // and exponents [sites]
     double2* full_a = nullptr;         // [V][12] label-ordered scratch
     double2* full_b = nullptr;
@@ -366,8 +366,16 @@ struct StencilArgs {
                              // the other callers' vectors matter by their norms
 };
 gs_status launch_stencil_f64(gs_ctx* c, const StencilArgs& a);
+// Whether memory is there for an array that only makes the FP64 stencils faster (they
+// run in double precision without it): an eighth of what is free, so that the
+// solvers' vectors, up to some 4 KB a site, still find room where they did before.
+inline bool fx_room(size_t bytes) {
+    size_t free = 0, total = 0;
+    return bytes < ((size_t)64 << 20) || (cudaMemGetInfo(&free, &total) == cudaSuccess && bytes <= free / 8);
+}
 // whether fixed point holds plan p's links: 1, 0, or -1 if the host does not know yet
 inline int plan_fits(const Plan* p) {
+    if (!p->fx_links) return 0;
     const unsigned w = *p->fit_host;
     return (w >> 1) != (p->fit_gen & 0x7fffffffu) ? -1 : !(w & 1u);
 }

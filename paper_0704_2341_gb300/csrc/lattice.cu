@@ -133,7 +133,8 @@ __global__ void k_count_hops(int64_t V, int64_t nb, const int2* __restrict__ nbr
 // and the same in fixed point, in groups of 32 labels (fx_index): a block turns
 // 32 sites around in shared memory so that both arrays are written in whole
 // lines.  *flag = 1 if an entry, or the sum of a row or a column, does not fit
-// fixed point (the stencils then use the double-precision links).
+// fixed point, or there is no room for it (fx null): the stencils then use the
+// double-precision links.
 __global__ void __launch_bounds__(256) k_pack_links(int64_t V, const int32_t* __restrict__ perm,
                                                     const double2* __restrict__ U, double2* __restrict__ links,
                                                     int4* __restrict__ fx, int* __restrict__ flag) {
@@ -145,11 +146,16 @@ __global__ void __launch_bounds__(256) k_pack_links(int64_t V, const int32_t* __
             const double2 u = U[(int64_t)perm[base + site] * 36 + k];
             const double2 l = make_double2(-0.5 * u.x, -0.5 * u.y);
             links[base * 36 + i] = l;
+            if (!fx) continue;
             const bool fits = fabs(l.x) <= kFxLinkMax && fabs(l.y) <= kFxLinkMax;   // false for NaN
             if (!fits) atomicExch(flag, 1);
             const FxLimb re = fx_split(fits ? __double2ll_rn(l.x * 0x1p61) : 0);
             const FxLimb im = fx_split(fits ? __double2ll_rn(l.y * 0x1p61) : 0);
             sm[site][k] = make_int4(re.lo, re.hi, im.lo, im.hi);
+        }
+        if (!fx) {
+            if (threadIdx.x == 0) atomicExch(flag, 1);
+            continue;
         }
         __syncthreads();
         for (int i = threadIdx.x; i < 36 * 32; i += 256) {
@@ -258,7 +264,6 @@ gs_status get_plan(gs_ctx* c, int type, int dir, int inverse, Plan** out) {
         cudaMalloc(&p->label, V * sizeof(int32_t)) != cudaSuccess ||
         cudaMalloc(&p->nbr, V * 4 * sizeof(int2)) != cudaSuccess ||
         cudaMalloc(&p->links, V * 36 * sizeof(double2)) != cudaSuccess ||
-        cudaMalloc(&p->fx_links, fx_padded(V) * 36 * sizeof(int4)) != cudaSuccess ||
         cudaMalloc(&p->fx_flag, sizeof(int)) != cudaSuccess ||
         cudaHostAlloc((void**)&p->fit_host, sizeof(unsigned), cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer((void**)&p->fit_dev, (void*)p->fit_host, 0) != cudaSuccess) {
@@ -268,6 +273,11 @@ gs_status get_plan(gs_ctx* c, int type, int dir, int inverse, Plan** out) {
                        (long long)V);
     }
     *p->fit_host = 0;
+    const size_t fx_bytes = (size_t)fx_padded(V) * 36 * sizeof(int4);
+    if (!fx_room(fx_bytes) || cudaMalloc(&p->fx_links, fx_bytes) != cudaSuccess) {
+        cudaGetLastError();
+        p->fx_links = nullptr;
+    }
     Dims d;
     for (int mu = 0; mu < 4; ++mu) d.L[mu] = c->dims[mu];
     const int g = grid_for(V, 256, c->num_sms * 8);

@@ -639,6 +639,7 @@ __global__ void __launch_bounds__(kT<NS>, NS) k_bicg_persistent_fx(const __grid_
 struct FxScratch {
     int64_t cap = 0;               // sites
     longlong2* m = nullptr;        // mantissas of p and of s
+    int64_t vec_cap = 0;           // sites of x and r, which the on-chip form does without
     double2 *x = nullptr, *r = nullptr;   // r: the right-hand side may be the inner workspace's own r
     unsigned* e = nullptr;         // exponent words of p and of s
     ulonglong2* rec = nullptr;
@@ -654,7 +655,7 @@ void free_persist_fx(gs_ctx* c) {
     c->persist_fx = nullptr;
 }
 
-static gs_status fx_scratch(gs_ctx* c, int64_t sites, FxScratch** out) {
+static gs_status fx_scratch(gs_ctx* c, int64_t sites, bool vectors, FxScratch** out) {
     FxScratch* f = (FxScratch*)c->persist_fx;
     if (f && f->cap < sites) {
         free_persist_fx(c);
@@ -665,7 +666,6 @@ static gs_status fx_scratch(gs_ctx* c, int64_t sites, FxScratch** out) {
         c->persist_fx = f;
         const size_t vec = (size_t)fx_padded(sites) * kSiteC * 16;
         if (cudaMalloc(&f->m, 2 * vec) != cudaSuccess ||
-            cudaMalloc(&f->x, vec) != cudaSuccess || cudaMalloc(&f->r, vec) != cudaSuccess ||
             cudaMalloc(&f->e, 2 * sites * sizeof(unsigned)) != cudaSuccess ||
             cudaMalloc(&f->rec, 2 * kFxMaxGrid * kFxRec * sizeof(ulonglong2)) != cudaSuccess ||
             cudaMalloc(&f->err, sizeof(int)) != cudaSuccess) {
@@ -674,6 +674,19 @@ static gs_status fx_scratch(gs_ctx* c, int64_t sites, FxScratch** out) {
             return set_err(c, GS_ENOMEM, "allocating the persistent solver's vectors failed");
         }
         f->cap = sites;
+    }
+    if (vectors && f->vec_cap < sites) {
+        const size_t vec = (size_t)fx_padded(sites) * kSiteC * sizeof(double2);
+        cudaFree(f->x);
+        cudaFree(f->r);
+        f->x = f->r = nullptr;
+        f->vec_cap = 0;
+        if (cudaMalloc(&f->x, vec) != cudaSuccess || cudaMalloc(&f->r, vec) != cudaSuccess) {
+            cudaGetLastError();
+            free_persist_fx(c);
+            return set_err(c, GS_ENOMEM, "allocating the persistent solver's vectors failed");
+        }
+        f->vec_cap = sites;
     }
     *out = f;
     return GS_OK;
@@ -725,8 +738,13 @@ static gs_status launch_fx_solver(gs_ctx* c, PArgsFx& P, const FxScratch* f) {
 gs_status persistent_bicg_fx(gs_ctx* c, const Plan* p, const StencilArgs& S, const double2* b, double2* x,
                              InnerWork& w, double tol, int maxit) {
     const int64_t n = S.n_out;
+    // A set with a tile for every SM at most keeps everything on chip; in a
+    // batched call of such sets only, with 8 warps a tile, so that two solves
+    // share an SM.
+    const bool small = c->coop_block_cap == 0 && n <= (int64_t)kSitesPerBlock * c->num_sms &&
+                       (!c->ledger || c->ledger->resident);
     FxScratch* f = nullptr;
-    gs_status s = fx_scratch(c, n, &f);
+    gs_status s = fx_scratch(c, n, !small, &f);
     if (s != GS_OK) return s;
     PArgsFx P;
     memset(&P, 0, sizeof P);
@@ -753,12 +771,8 @@ gs_status persistent_bicg_fx(gs_ctx* c, const Plan* p, const StencilArgs& S, con
     P.wait_ns = c->wait_ns ? c->wait_ns : kWaitNs;
     P.st = w.st;
     P.phases = c->prof.on ? c->prof.phases_dev : nullptr;
-    // A set with a tile for every SM at most keeps everything on chip; in a
-    // batched call of such sets only, with 8 warps a tile, so that two solves
-    // share an SM.
-    const bool small = c->coop_block_cap == 0 && n <= (int64_t)kSitesPerBlock * c->num_sms;
-    if (!c->ledger) return small ? launch_fx_solver<1, true>(c, P, f) : launch_fx_solver<2, false>(c, P, f);
-    return small && c->ledger->resident ? launch_fx_solver<2, true>(c, P, f) : launch_fx_solver<2, false>(c, P, f);
+    if (!small) return launch_fx_solver<2, false>(c, P, f);
+    return c->ledger ? launch_fx_solver<2, true>(c, P, f) : launch_fx_solver<1, true>(c, P, f);
 }
 
 }  // namespace gs

@@ -167,11 +167,12 @@ gs_status inner_solve_f64(gs_ctx* c, const Plan* p, const double2* t, double2* z
             GS_CUDA(c, cudaEventSynchronize(w.ev[0]));
             return GS_OK;
         };
-        const bool fits = plan_fits(p) != 0;
+        bool fits = plan_fits(p) != 0;
         if (fits) {
             s = persistent_bicg_fx(c, p, k1, t, z, w, o.inner_tol, o.inner_max_iter);
-            if (s != GS_OK || (s = finished()) != GS_OK) return s;
-            ledger_release(c);
+            if (s == GS_ENOMEM) fits = false;     // the double-precision solver needs no vectors of its own
+            else if (s != GS_OK || (s = finished()) != GS_OK) return s;
+            else ledger_release(c);
         }
         if (!fits || pub->status == kFxUnfit || pub->status == GS_BREAKDOWN) {
             s = persistent_bicg_f64(c, k1, k3, t, z, w, n, o.inner_tol, o.inner_max_iter);

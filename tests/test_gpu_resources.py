@@ -144,3 +144,36 @@ def test_batched_fp64_solves(env, dims, fields):
         # as many launches as alone, up to an outer iteration or two (19 launches at most)
         assert st.kernel_launches <= one.kernel_launches + 40
         c.close()
+
+
+def test_lattice_that_just_fits(env):
+    """The fixed-point copies are there for speed only: with room for what double
+    precision needs (1768 bytes a site) and not for them, the calls run in double
+    precision."""
+    torch, gs = env
+    dims, m0 = (16, 16, 16, 32), 0.1
+    V = li.volume(dims)
+    rng = np.random.default_rng(10)
+    U = to_dev(li.random_gauge(dims, 0.3, 60), torch)
+    x = to_dev(rng.standard_normal((V, 12)) + 1j * rng.standard_normal((V, 12)), torch)
+    xb = x[:V // 16].clone()
+    out = []
+    torch.cuda.synchronize()
+    for tight in (False, True):
+        torch.cuda.empty_cache()
+        y, yb = torch.empty_like(x), torch.empty_like(xb)
+        hog = None
+        if tight:
+            hog = torch.empty(torch.cuda.mem_get_info()[0] - (1768 * V + (32 << 20)), dtype=torch.uint8, device="cuda:0")
+        ctx = gs.Context(dims, m0, torch.cuda.current_stream().cuda_stream)
+        ctx.set_gauge(U)
+        ctx.wilson_apply(x, y)
+        del hog
+        torch.cuda.empty_cache()
+        ctx.schur_apply(1, 0, 0, xb, yb, gs.gs_default_opts(inner_tol=1e-12))
+        torch.cuda.synchronize()
+        ctx.close()
+        out.append((y, yb))
+    (y1, b1), (y2, b2) = out
+    assert (y1 - y2).abs().max() <= 1.5e-13 * x.abs().max()
+    assert (b1 - b2).norm() <= 1e-10 * b1.norm()
