@@ -169,7 +169,8 @@ enum { GS_OPT_STENCIL_VARIANT = 1, GS_OPT_INNER_KERNEL = 2, GS_OPT_NET_KERNEL = 
  * GS_OPT_COOP_BLOCKS: the number of blocks the persistent (cooperative)
  * solver kernels of this problem use while schur_solve_batched runs several
  * solves at once (the caller then keeps their sum within what the GPU holds
- * at once); 0 = granted at each launch by the call's block ledger (the
+ * at once: 3 per SM; the fixed-point FP64 solver takes two larger blocks
+ * for three); 0 = granted at each launch by the call's block ledger (the
  * default): FP64 inner solves of a call whose rest sets all have at most 32
  * sites per SM take a block per 32-site tile, others an even share of the
  * co-resident blocks among the running solves; FP32 / BF16 about 96 sites per

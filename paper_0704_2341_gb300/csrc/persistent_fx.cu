@@ -705,7 +705,10 @@ static gs_status launch_fx_solver(gs_ctx* c, PArgsFx& P, const FxScratch* f) {
     const int64_t tiles = (P.n + kSitesPerBlock - 1) / kSitesPerBlock;
     int64_t g = (int64_t)per_sm * c->num_sms;
     if (c->coop_block_cap > 0) {
-        if (g > c->coop_block_cap) g = c->coop_block_cap;
+        // GS_OPT_COOP_BLOCKS counts thirds of an SM, two blocks here take what three of
+        // the double-precision solver's did: counts that fit the GPU together still do
+        const int64_t cap = (int64_t)c->coop_block_cap * 2 / 3;
+        if (g > cap) g = cap > 0 ? cap : 1;
     } else if (c->ledger) {
         const int64_t usable = ledger_capacity(per_sm, c->num_sms);
         const int64_t n = c->ledger->running.load() > 1 ? c->ledger->running.load() : 1;

@@ -177,3 +177,23 @@ def test_lattice_that_just_fits(env):
     (y1, b1), (y2, b2) = out
     assert (y1 - y2).abs().max() <= 1.5e-13 * x.abs().max()
     assert (b1 - b2).norm() <= 1e-10 * b1.norm()
+
+
+def test_block_counts_that_fill_the_gpu(env):
+    """GS_OPT_COOP_BLOCKS: four FP64 solves with a quarter of 3 blocks per SM each, which is what
+    the GPU holds by the option's description, run together."""
+    torch, gs = env
+    dims = (8, 8, 8, 8)
+    blocks = 3 * torch.cuda.get_device_properties(0).multi_processor_count // 4
+    streams = [torch.cuda.Stream() for _ in range(4)]
+    ctxs = [_ctx(gs, torch, dims, 0.0, li.random_gauge(dims, 0.3, 70 + k), s.cuda_stream) for k, s in enumerate(streams)]
+    probs = []
+    for k, c in enumerate(ctxs):
+        c.set_option(gs.GS_OPT_COOP_BLOCKS, blocks)
+        f = to_dev(li.gaussian_source(dims, 80 + k), torch)
+        probs.append(dict(ctx=c.handle, type=1 + k % 2, dir=0, inverse=0, nrhs=1, f=f, x=torch.zeros_like(f)))
+    torch.cuda.synchronize()
+    status, stats = gs.schur_solve_batched(probs, gs.gs_default_opts())
+    assert status == gs.GS_OK and max(st.true_residual for st in stats) <= 1e-10
+    for c in ctxs:
+        c.close()
