@@ -129,8 +129,12 @@ int64_t ledger_grant(gs_ctx* c, int64_t capacity, int64_t want, int64_t target, 
     for (auto& e : L->held)
         if (e.ctx == c) mine = &e;
     if (!mine) return 0;
-    const auto t0 = std::chrono::steady_clock::now();
-    const auto bound = std::chrono::nanoseconds((long long)(c->wait_ns > 0 ? c->wait_ns : 1000000000ull) * 60);
+    if (least > capacity) return 0;
+    // Waiting is ordinary here (the FP64 solver's grids are granted whole) and as long
+    // as the other solves take, so nothing limits it, the device-side wait limit
+    // least of all.  It ends: a grant needs no more than the others leave free, their
+    // kernels end by themselves (every device-side wait is bounded), and a
+    // solve that waits holds no more than it was granted, so one of them can go on.
     for (;;) {
         // held: blocks that may be in flight now; claimed: the same with
         // every solve that has not launched yet counted at the reserve
@@ -150,7 +154,6 @@ int64_t ledger_grant(gs_ctx* c, int64_t capacity, int64_t want, int64_t target, 
         }
         // every block is held by the others' kernels in flight: one of them
         // ends or shrinks at its next launch
-        if (std::chrono::steady_clock::now() - t0 > bound) return 0;
         L->cv.wait_for(lk, std::chrono::milliseconds(1));
         for (auto& e : L->held)
             if (e.ctx == c) mine = &e;

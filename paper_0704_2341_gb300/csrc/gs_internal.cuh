@@ -216,8 +216,8 @@ struct BlockLedger {
 void ledger_enter(BlockLedger* L, const gs_ctx* c);
 void ledger_leave(BlockLedger* L, const gs_ctx* c);
 // blocks for c's next cooperative grid out of `capacity`: at most want and
-// target, at least `least`, never more than the others leave free; 0 if they
-// did not become free within the context's wait limit x 60
+// target, at least `least`, never more than the others leave free (it waits until they
+// are); 0 if `least` is more than there is
 int64_t ledger_grant(gs_ctx* c, int64_t capacity, int64_t want, int64_t target, int64_t least = 1);
 // The blocks of one FP64 batched call: those of the fixed-point solver that are
 // co-resident at per_sm an SM, less some slots for the other solves' small kernels.

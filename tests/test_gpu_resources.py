@@ -197,3 +197,24 @@ def test_block_counts_that_fill_the_gpu(env):
     assert status == gs.GS_OK and max(st.true_residual for st in stats) <= 1e-10
     for c in ctxs:
         c.close()
+
+
+def test_waiting_for_blocks_is_no_timeout(env):
+    """24 FP64 solves at once on 8^4 wait tens of milliseconds for their turn; the wait limit of
+    the kernels (1 ms here) has nothing to do with it."""
+    torch, gs = env
+    dims, N = (8, 8, 8, 8), 24
+    U = li.random_gauge(dims, 0.3, 90)
+    streams = [torch.cuda.Stream() for _ in range(N)]
+    ctxs = [_ctx(gs, torch, dims, 0.0, U, s.cuda_stream) for s in streams]
+    ctxs[0].set_option(gs.GS_OPT_BATCH_LANES, N)
+    probs = []
+    for k, c in enumerate(ctxs):
+        c.set_option(gs.GS_OPT_WAIT_LIMIT_US, 1000)
+        f = to_dev(li.gaussian_source(dims, 100 + k), torch)
+        probs.append(dict(ctx=c.handle, type=1, dir=0, inverse=k % 2, nrhs=1, f=f, x=torch.zeros_like(f)))
+    torch.cuda.synchronize()
+    status, stats = gs.schur_solve_batched(probs, gs.gs_default_opts())
+    assert status == gs.GS_OK and max(st.true_residual for st in stats) <= 1e-10
+    for c in ctxs:
+        c.close()
