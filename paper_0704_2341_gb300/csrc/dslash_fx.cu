@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(kFxThreads<NS>, NS) k_dslash_fx(const __grid_c
     if (skip) return;
     const bool links_bad = __ldg(a.fxflag) != 0;
     double e[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    fx_stencil<EPI, false, NS, KEEP>(a, kSitesPerBlock, links_bad, sm, sE, redo, l, e);
+    fx_stencil<EPI, NS, KEEP>(a, links_bad, sm, sE, redo, l, e);
     stencil_finish<EPI, kFxThreads<NS>>(a, e);
 }
 

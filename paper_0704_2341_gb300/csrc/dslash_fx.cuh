@@ -49,7 +49,7 @@ __device__ __forceinline__ int fx_partner(int w, int s) { return ((w < 8) != (s 
 // running when this one starts (programmatic launch), so they are not constant
 // for this kernel's lifetime, as __ldg would have it, and only a plain load stays
 // behind griddepcontrol.wait.
-template <int NS, bool CG>
+template <int NS>
 __device__ __forceinline__ void fx_load_spinor(const StencilArgs& a, int w, int in, FxOperands<NS>& o) {
     const longlong2* p = a.fxm + fx_index(in, kSiteC);
 #pragma unroll
@@ -59,8 +59,8 @@ __device__ __forceinline__ void fx_load_spinor(const StencilArgs& a, int w, int 
         const longlong2* pq = p + fx_partner(w, s) * 32;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            o.s[k][c] = CG ? __ldcg(ps + c * 32) : ps[c * 32];
-            o.q[k][c] = CG ? __ldcg(pq + c * 32) : pq[c * 32];
+            o.s[k][c] = ps[c * 32];
+            o.q[k][c] = pq[c * 32];
         }
     }
 }
@@ -129,22 +129,17 @@ __device__ __forceinline__ void fx_hop(const FxOperands<NS>& o, int w, int sh, F
 }
 
 // Epilogue dots of one complex output (see f64_tile).
-template <int EPI, bool CG>
+template <int EPI>
 __device__ __forceinline__ void stencil_dots(const StencilArgs& a, int64_t i, double re, double im, double (&e)[5]) {
     if (EPI == EPI_DOT_RHAT_V) {
-        const double2 rv = CG ? __ldcg(a.epi_vec + i) : a.epi_vec[i];
+        const double2 rv = a.epi_vec[i];
         e[0] = fma(rv.x, re, fma(rv.y, im, e[0]));
         e[1] = fma(rv.x, im, fma(-rv.y, re, e[1]));
-    } else if (EPI == EPI_DOT_TS || EPI == EPI_DOT_TSR) {
-        const double2 sv = CG ? __ldcg(a.epi_vec + i) : a.epi_vec[i];
+    } else if (EPI == EPI_DOT_TS) {
+        const double2 sv = a.epi_vec[i];
         e[0] = fma(re, sv.x, fma(im, sv.y, e[0]));
         e[1] = fma(re, sv.y, fma(-im, sv.x, e[1]));
         e[2] = fma(re, re, fma(im, im, e[2]));
-        if (EPI == EPI_DOT_TSR) {
-            const double2 rv = CG ? __ldcg(a.epi_vec2 + i) : a.epi_vec2[i];
-            e[3] = fma(rv.x, re, fma(rv.y, im, e[3]));
-            e[4] = fma(rv.x, im, fma(-rv.y, re, e[4]));
-        }
     }
 }
 
@@ -207,11 +202,10 @@ __device__ __forceinline__ int fx_label(const StencilArgs& a, int64_t base, int 
 
 // Exponent word of the input site with label l (kFxZero outside the input
 // range) and its index.
-template <bool CG>
 __device__ __forceinline__ int fx_site(const StencilArgs& a, int l, unsigned& i) {
     i = l < 0 ? 0xffffffffu : (unsigned)l - (unsigned)a.a0;   // labels below the range wrap above it
     if (i >= (unsigned)a.fxn) return kFxZero;
-    return CG ? __ldcg(a.fxe + i) : a.fxe[i];
+    return a.fxe[i];
 }
 
 // Whether the inputs of a spin component's hops are zero: what fixed point then gives
@@ -247,14 +241,14 @@ __device__ __forceinline__ bool fx_weak(const FxShared& sm, const int (&sE)[8][k
     return hops > 0 && top < 1 << (fx_weak_bits(hops) - 32);
 }
 
-// One tile of ts <= 32 output sites from base, l = fx_label of this tile.
+// One tile of up to 32 output sites from base, l = fx_label of this tile.
 // Phase 1: a warp per hop (and spin component).  Phase 2: three warps per spin
 // component, a thread one complex output: sum of the hops, conversion,
 // diagonal, addend and the epilogue dots.  Returns true if the tile has to be done
 // in double precision: an input site does not fit fixed point (nothing is written), or
 // with KEEP a component is weak.  The output is not the addend.
-template <int EPI, bool CG, int NS, bool KEEP>
-__device__ __forceinline__ bool fx_tile(const StencilArgs& a, int64_t base, int ts, int l, FxShared& sm,
+template <int EPI, int NS, bool KEEP>
+__device__ __forceinline__ bool fx_tile(const StencilArgs& a, int64_t base, int l, FxShared& sm,
                                         int (&sE)[8][kSitesPerBlock], double (&e)[5]) {
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -262,10 +256,10 @@ __device__ __forceinline__ bool fx_tile(const StencilArgs& a, int64_t base, int 
     bool bad;
     {
         unsigned i;
-        const int x = fx_site<CG>(a, l, i);
+        const int x = fx_site(a, l, i);
         FxOperands<NS> o;
         if (i < (unsigned)a.fxn) {
-            fx_load_spinor<NS, CG>(a, w, (int)i, o);
+            fx_load_spinor<NS>(a, w, (int)i, o);
             fx_load_link<NS>(a, w, (w & 2) ? l : (int)(a.o0 + base) + lane, o);
         }
         bad = x < 0;
@@ -289,7 +283,7 @@ __device__ __forceinline__ bool fx_tile(const StencilArgs& a, int64_t base, int 
         const int spin = v / 3;
         const int i = (v - 3 * spin) * 32 + lane;
         const int site = i / 3, c = i - 3 * site;
-        if (site >= ts || base + site >= a.n_out) continue;
+        if (base + site >= a.n_out) continue;
         const I2 t = fx_sum(sm, site, spin, c);
         int E = 0;
 #pragma unroll
@@ -303,7 +297,7 @@ __device__ __forceinline__ bool fx_tile(const StencilArgs& a, int64_t base, int 
         const int64_t o = (base + site) * kSiteC + k;
         double re = fx_to_double(t.x, E), im = fx_to_double(t.y, E);
         if (self) {
-            const double2 sv = CG ? __ldcg(self) : __ldg(self);
+            const double2 sv = __ldg(self);
             re = fma(a.diag, sv.x, re);
             im = fma(a.diag, sv.y, im);
         }
@@ -312,12 +306,12 @@ __device__ __forceinline__ bool fx_tile(const StencilArgs& a, int64_t base, int 
             im = -im;
         }
         if (a.addend) {
-            const double2 av = CG ? __ldcg(a.addend + o) : a.addend[o];
+            const double2 av = a.addend[o];
             re += av.x;
             im += av.y;
         }
         a.out[o] = make_double2(re, im);
-        stencil_dots<EPI, CG>(a, o, re, im, e);
+        stencil_dots<EPI>(a, o, re, im, e);
     }
     if (KEEP) {
         if (!__syncthreads_or(weak)) return false;
@@ -339,19 +333,19 @@ constexpr int kFxRedoWords = 640;
 // them when a link does not fit) are done in double precision afterwards, so
 // that the rare path costs the common one no registers.  With KEEP `redo` holds them, as
 // the hops' sums are gone by then.
-template <int EPI, bool CG, int NS, bool KEEP>
-__device__ __forceinline__ void fx_stencil(const StencilArgs& a, int ts, bool links_bad, FxShared& sm,
+template <int EPI, int NS, bool KEEP>
+__device__ __forceinline__ void fx_stencil(const StencilArgs& a, bool links_bad, FxShared& sm,
                                            int (&sE)[8][kSitesPerBlock], unsigned* redo, int l, double (&e)[5]) {
-    const int64_t step = (int64_t)gridDim.x * ts;
+    const int64_t step = (int64_t)gridDim.x * kSitesPerBlock;
     const int w = (threadIdx.x >> 5) * NS;
     bool any = links_bad;
     if constexpr (KEEP) {
         for (int i = threadIdx.x; i < kFxRedoWords; i += kFxThreads<NS>) redo[i] = links_bad ? ~0u : 0u;
         int tile = 0;
         if (!links_bad)
-            for (int64_t base = (int64_t)blockIdx.x * ts; base < a.n_out; base += step, ++tile) {
-                const int next = fx_label(a, base + step, ts, w);
-                if (fx_tile<EPI, CG, NS, true>(a, base, ts, l, sm, sE, e)) {
+            for (int64_t base = (int64_t)blockIdx.x * kSitesPerBlock; base < a.n_out; base += step, ++tile) {
+                const int next = fx_label(a, base + step, kSitesPerBlock, w);
+                if (fx_tile<EPI, NS, true>(a, base, l, sm, sE, e)) {
                     any = true;
                     if (threadIdx.x == 0) redo[tile >> 5] |= 1u << (tile & 31);
                 }
@@ -360,22 +354,22 @@ __device__ __forceinline__ void fx_stencil(const StencilArgs& a, int ts, bool li
         if (any) {
             __syncthreads();
             tile = 0;
-            for (int64_t base = (int64_t)blockIdx.x * ts; base < a.n_out; base += step, ++tile)
-                if (redo[tile >> 5] >> (tile & 31) & 1u) f64_tile<EPI, CG>(a, base, ts, sm.f64, e);
+            for (int64_t base = (int64_t)blockIdx.x * kSitesPerBlock; base < a.n_out; base += step, ++tile)
+                if (redo[tile >> 5] >> (tile & 31) & 1u) f64_tile<EPI>(a, base, kSitesPerBlock, sm.f64, e);
         }
         return;
     }
     if (!links_bad)
-        for (int64_t base = (int64_t)blockIdx.x * ts; base < a.n_out; base += step) {
-            const int next = fx_label(a, base + step, ts, w);
-            any |= fx_tile<EPI, CG, NS, false>(a, base, ts, l, sm, sE, e);
+        for (int64_t base = (int64_t)blockIdx.x * kSitesPerBlock; base < a.n_out; base += step) {
+            const int next = fx_label(a, base + step, kSitesPerBlock, w);
+            any |= fx_tile<EPI, NS, false>(a, base, l, sm, sE, e);
             l = next;
         }
     if (any)
-        for (int64_t base = (int64_t)blockIdx.x * ts; base < a.n_out; base += step) {
+        for (int64_t base = (int64_t)blockIdx.x * kSitesPerBlock; base < a.n_out; base += step) {
             unsigned i;
-            const bool bad = fx_site<CG>(a, fx_label(a, base, ts, w), i) < 0;
-            if (__syncthreads_or(bad) || links_bad) f64_tile<EPI, CG>(a, base, ts, sm.f64, e);
+            const bool bad = fx_site(a, fx_label(a, base, kSitesPerBlock, w), i) < 0;
+            if (__syncthreads_or(bad) || links_bad) f64_tile<EPI>(a, base, kSitesPerBlock, sm.f64, e);
         }
 }
 

@@ -517,11 +517,8 @@ __device__ __forceinline__ void site_dir(const LpArgs& a, int64_t k, int2 nb, fl
 }
 
 // Raw (still packed) operands of one direction of one site: the two
-// neighbour spinors and the two links, as loaded; unpacked only when used.
-template <class S>
-struct Raw;
-template <>
-struct Raw<float> {
+// neighbour spinors and the two links, as loaded (FP32); unpacked only when used.
+struct Raw {
     float4 pf[6], pb[6], lf[3], lb[3];
     __device__ __forceinline__ void load(const LpArgs& a, int mu, int64_t jf, int64_t jb, int64_t k) {
         const float4* in = (const float4*)a.in;
@@ -555,8 +552,8 @@ struct Raw<float> {
     }
 };
 // the two hops of direction MU from raw operands (masked hops contribute 0)
-template <class S, int MU>
-__device__ __forceinline__ void raw_dir(const Raw<S>& r, bool hf, bool hb, float (&acc)[24]) {
+template <int MU>
+__device__ __forceinline__ void raw_dir(const Raw& r, bool hf, bool hb, float (&acc)[24]) {
     float pf[24], pb[24], lf[12], lb[12];
     r.unpack(pf, pb, lf, lb);
     if (hf) {
@@ -595,12 +592,13 @@ __device__ __forceinline__ void raw_dir(const Raw<S>& r, bool hf, bool hb, float
 template <class S, int EPI>
 __device__ __forceinline__ void lp_finish(const LpArgs& a, LpState* st, float (&tot)[3]);
 
-// Variant "pipelined site": one thread per site, like "site", but the loads of
+// Variant "pipelined site" (FP32 storage): one thread per site, like "site", but the loads of
 // direction mu + 1 are issued before direction mu is computed (two operand
 // buffers in registers, kept packed until used), so each thread waits for
 // memory about twice per site instead of five times; fewer blocks fit per SM.
-template <class S, int EPI, int MINB>
+template <int EPI, int MINB>
 __global__ void __launch_bounds__(128, MINB) k_dslash_lp_pipe(LpArgs a) {
+    using S = float;
     const bool skip = a.st != nullptr && a.st->done;
     if (a.ran != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *a.ran = skip ? 0 : 1;
     if (skip) return;
@@ -612,20 +610,20 @@ __global__ void __launch_bounds__(128, MINB) k_dslash_lp_pipe(LpArgs a) {
         // out-of-set neighbours (-1) read the site itself and are masked
         const bool h0f = n01.x >= 0, h0b = n01.y >= 0, h1f = n01.z >= 0, h1b = n01.w >= 0;
         const bool h2f = n23.x >= 0, h2b = n23.y >= 0, h3f = n23.z >= 0, h3b = n23.w >= 0;
-        Raw<S> r0, r1;
+        Raw r0, r1;
         r0.load(a, 0, h0f ? n01.x : k, h0b ? n01.y : k, k);
         r1.load(a, 1, h1f ? n01.z : k, h1b ? n01.w : k, k);
         float acc[24];
 #pragma unroll
         for (int q = 0; q < 24; ++q) acc[q] = 0.f;
-        raw_dir<S, 0>(r0, h0f, h0b, acc);
+        raw_dir<0>(r0, h0f, h0b, acc);
         r0.load(a, 2, h2f ? n23.x : k, h2b ? n23.y : k, k);
-        raw_dir<S, 1>(r1, h1f, h1b, acc);
+        raw_dir<1>(r1, h1f, h1b, acc);
         r1.load(a, 3, h3f ? n23.z : k, h3b ? n23.w : k, k);
-        raw_dir<S, 2>(r0, h2f, h2b, acc);
+        raw_dir<2>(r0, h2f, h2b, acc);
         float self[24];
         Store<S>::load_spinor(a.in, a.n, k, self);
-        raw_dir<S, 3>(r1, h3f, h3b, acc);
+        raw_dir<3>(r1, h3f, h3b, acc);
 #pragma unroll
         for (int q = 0; q < 24; ++q) acc[q] = fmaf(a.diag, self[q], acc[q]);
         Store<S>::store_spinor(a.out, a.n, k, acc);

@@ -335,10 +335,10 @@ gs_status launch_lp_stencil(gs_ctx* c, LpArgs a, long long hops, int variant, lo
         }
 #define GS_PIPE_LAUNCH(MB)                                                                       \
         switch (a.epi) {                                                                         \
-            case EPI_NONE: k_dslash_lp_pipe<S, EPI_NONE, MB><<<(int)g, b, 0, c->stream>>>(a); break; \
+            case EPI_NONE: k_dslash_lp_pipe<EPI_NONE, MB><<<(int)g, b, 0, c->stream>>>(a); break; \
             case EPI_DOT_RHAT_V:                                                                 \
-                k_dslash_lp_pipe<S, EPI_DOT_RHAT_V, MB><<<(int)g, b, 0, c->stream>>>(a); break;  \
-            default: k_dslash_lp_pipe<S, EPI_DOT_TS, MB><<<(int)g, b, 0, c->stream>>>(a); break; \
+                k_dslash_lp_pipe<EPI_DOT_RHAT_V, MB><<<(int)g, b, 0, c->stream>>>(a); break;  \
+            default: k_dslash_lp_pipe<EPI_DOT_TS, MB><<<(int)g, b, 0, c->stream>>>(a); break; \
         }
         if (variant == 3) {
             GS_SITE_LAUNCH(6)
