@@ -1073,6 +1073,9 @@ def main():
         "achieved_definition": "algorithmic flops of all the family's launches in the timed steps / the "
                                "union of their CUDA-event intervals (the four permutations' solver "
                                "launches run concurrently, %.2f at a time on average)" % concurrency,
+        "frac_definition": "algorithmic FP64 flops against what the FP64 pipe could do; the hops run as "
+                           "integer multiply-adds (block fixed point), so this is no pipe's utilisation "
+                           "and may pass 1",
         "launches": prof[dom]["launches"], "avg_launch_us": 1e3 * avg_ms,
         "per_launch_achieved_tflops": flops_per_launch / (avg_ms / 1e3) / 1e12 if avg_ms > 0 else 0.0,
         "algorithmic_flops_per_launch": flops_per_launch,

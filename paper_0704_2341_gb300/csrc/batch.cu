@@ -14,10 +14,11 @@
 // solve alone, 5.49 / 5.31 / 5.26 / 5.32 s with 2 / 3 / 4 / 6 at once, so four
 // lanes by default).  The cooperative grids of the running solves are drawn
 // from one block ledger (BlockLedger): all cooperative blocks of a call have one
-// size (its inner precision and the sizes of its lattices pick one kernel), a
-// grid is granted only from blocks no other solve holds, so all of them stay
-// co-resident, and the blocks a finished solve frees go to the next launches of
-// the others.  On small lattices the FP64 solver's blocks keep their tile on
+// size (its inner precision and the sizes of its lattices pick one kernel; those of
+// the double-precision solver, for what fixed point cannot hold, are smaller and
+// count as one each), a grid is granted only from blocks no other solve holds, so
+// all of them stay co-resident, and the blocks a finished solve frees go to the
+// next launches of the others.  On small lattices the FP64 solver's blocks keep their tile on
 // chip and are granted a whole grid at a time; a finished launch gives them back
 // at once (four permutations of 8^4: 126 ms against 154 with even shares of
 // blocks that keep their vectors in memory).
@@ -217,8 +218,7 @@ gs_status schur_solve_batched(int nprob, gs_ctx* const* ctxs, const int* type, c
     for (auto& s : sts) memset(&s, 0, sizeof s);
     std::vector<std::string> msg(nprob);
     BlockLedger ledger;
-    // a solve that has not launched yet is counted at a third of an even
-    // share of the co-resident blocks (one block per SM share at 3 per SM)
+    // a solve that has not launched yet is counted at its share of one block per SM
     ledger.reserve = std::max(1, ctxs[0]->num_sms / std::max(1, lanes));
     // the on-chip FP64 solver's grids are granted whole: the largest rest set
     // (15/16 of a lattice, Type I) has to leave room for another solve

@@ -191,7 +191,8 @@ struct gs_ctx;
 
 namespace gs {
 // The blocks of the persistent solver kernels of one schur_solve_batched
-// call.  In one call those blocks all have one size, so they are
+// call.  In one call those blocks all have one size (the double-precision FP64
+// solver's are smaller than the fixed-point one's and count as one), so they are
 // interchangeable and the GPU holds per_sm x SMs of them at once.
 // held[] records, per running solve, the blocks its kernel may have in
 // flight: its last grid (its previous kernel has finished before it launches
