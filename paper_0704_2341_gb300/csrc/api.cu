@@ -107,7 +107,10 @@ gs_status gs_create(gs_ctx** out, const int dims[4], double m0, void* stream) {
               cudaMalloc(&c->scal_dev, 64 * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&c->red.partial, kRedScratchDoubles * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&c->red.counter, sizeof(unsigned int)) == cudaSuccess &&
-              cudaHostAlloc(&c->scal_host, 64 * sizeof(double), 0) == cudaSuccess;
+              cudaHostAlloc(&c->scal_host, 64 * sizeof(double) + kMaxPlans * sizeof(unsigned), cudaHostAllocMapped) ==
+                  cudaSuccess &&
+              cudaHostGetDevicePointer((void**)&c->fit_dev, c->scal_host + 64, 0) == cudaSuccess;
+    c->fit_host = (volatile unsigned*)(c->scal_host + 64);
     if (!ok) {
         cudaGetLastError();
         gs_destroy(c);

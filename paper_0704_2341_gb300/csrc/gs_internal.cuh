@@ -106,6 +106,7 @@ __device__ __forceinline__ void publish(BicgState* st) {
 // ---------------------------------------------------------------------------
 // a permutation plan: label order, neighbour table and label-ordered links
 // ---------------------------------------------------------------------------
+constexpr int kMaxPlans = 16;   // the identity, two of Type I, eight of Type II
 struct Plan {
     int type = 0;          // 0 = identity (site order), GS_TYPE_I, GS_TYPE_II
     int dir = 0;
@@ -117,8 +118,8 @@ struct Plan {
     double2* links = nullptr;    // [V][4][9] -1/2 U_mu(perm[j]) in label order
     int4* fx_links = nullptr;    // the same in fixed point (fx.cuh): limbs (re.lo, re.hi, im.lo, im.hi); null: no room
     int* fx_flag = nullptr;      // device: 1 if a link lies outside fixed point's range
-    volatile unsigned* fit_host = nullptr;   // the same for the host, in mapped memory: 2 fit_gen + fx_flag once the
-    unsigned* fit_dev = nullptr;             // links of generation fit_gen are packed
+    volatile unsigned* fit_host = nullptr;   // the same for the host, in pinned memory (a word of the context's): 2 fit_gen +
+                                             // fx_flag once the links of generation fit_gen are packed
     unsigned fit_gen = 0;
     bool links_ready = false;
     long long hops[2][2] = {{0, 0}, {0, 0}};  // [out set][in set] in-set neighbour terms (0 = b, 1 = r)
@@ -245,7 +246,9 @@ struct gs_ctx {
     double2* full_b = nullptr;
     double2* full_c = nullptr;
     double* scal_dev = nullptr;        // small device scratch for norms
-    double* scal_host = nullptr;       // pinned
+    double* scal_host = nullptr;       // pinned: 64 doubles, then
+    volatile unsigned* fit_host = nullptr;   // the plans' words (Plan::fit_host),
+    unsigned* fit_dev = nullptr;             // and the same for the device
     gs::RedScratch red;
     long long launches = 0;
     long long stencil_sites = 0;

@@ -214,7 +214,6 @@ void free_plan(Plan* p) {
     cudaFree(p->links);
     cudaFree(p->fx_links);
     cudaFree(p->fx_flag);
-    if (p->fit_host) cudaFreeHost((void*)p->fit_host);
     cudaFree(p->dtinv);
     delete p;
 }
@@ -224,7 +223,7 @@ gs_status pack_plan_links(gs_ctx* c, Plan* p) {
     GS_CUDA(c, cudaMemsetAsync(p->fx_flag, 0, sizeof(int), c->stream));
     k_pack_links<<<grid_for(c->V, 32, c->num_sms * 16), 256, 0, c->stream>>>(c->V, p->perm, c->U_abi, p->links,
                                                                             p->fx_links, p->fx_flag);
-    k_publish_fit<<<1, 1, 0, c->stream>>>(p->fx_flag, ++p->fit_gen, p->fit_dev);
+    k_publish_fit<<<1, 1, 0, c->stream>>>(p->fx_flag, ++p->fit_gen, c->fit_dev + (p->fit_host - c->fit_host));
     c->launches += 2;
     GS_CHECK_LAUNCH(c);
     p->links_ready = true;
@@ -264,14 +263,13 @@ gs_status get_plan(gs_ctx* c, int type, int dir, int inverse, Plan** out) {
         cudaMalloc(&p->label, V * sizeof(int32_t)) != cudaSuccess ||
         cudaMalloc(&p->nbr, V * 4 * sizeof(int2)) != cudaSuccess ||
         cudaMalloc(&p->links, V * 36 * sizeof(double2)) != cudaSuccess ||
-        cudaMalloc(&p->fx_flag, sizeof(int)) != cudaSuccess ||
-        cudaHostAlloc((void**)&p->fit_host, sizeof(unsigned), cudaHostAllocMapped) != cudaSuccess ||
-        cudaHostGetDevicePointer((void**)&p->fit_dev, (void*)p->fit_host, 0) != cudaSuccess) {
+        cudaMalloc(&p->fx_flag, sizeof(int)) != cudaSuccess || c->plans.size() >= kMaxPlans) {
         free_plan(p);
         cudaGetLastError();
         return set_err(c, GS_ENOMEM, "allocating a permutation plan for V = %lld failed",
                        (long long)V);
     }
+    p->fit_host = c->fit_host + c->plans.size();
     *p->fit_host = 0;
     const size_t fx_bytes = (size_t)fx_padded(V) * 36 * sizeof(int4);
     if (!fx_room(fx_bytes) || cudaMalloc(&p->fx_links, fx_bytes) != cudaSuccess) {
