@@ -208,26 +208,6 @@ __device__ __forceinline__ int fx_site(const StencilArgs& a, int l, unsigned& i)
     return a.fxe[i];
 }
 
-// Whether the inputs of a spin component's hops are zero: what fixed point then gives
-// for it, zero, is exact.  j: the site's label.
-__device__ __forceinline__ bool fx_silent(const StencilArgs& a, int64_t j, int spin) {
-#pragma unroll 1
-    for (int q = 0; q < 8; ++q) {
-        const int2 n = __ldg(a.nbr + j * 4 + (q >> 1));
-        const int64_t l = (q & 1) ? n.y : n.x;
-        const double2* p = l >= a.a0 && l < a.a1 ? a.inA + (l - a.a0) * kSiteC
-                           : l >= a.a1 && l < a.b1 ? a.inB + (l - a.a1) * kSiteC : nullptr;
-        if (!p) continue;
-        const int up = spin < 2 ? spin : q < 4 ? 3 - spin : spin - 2;       // upper spin of the hop's row, and its partner
-        const int lo = q < 4 ? 3 - up : 2 + up;
-#pragma unroll 1
-        for (int c = 0; c < 3; ++c) {
-            const double2 s = __ldg(p + 3 * up + c), t = __ldg(p + 3 * lo + c);
-            if (s.x != 0.0 || s.y != 0.0 || t.x != 0.0 || t.y != 0.0) return false;
-        }
-    }
-    return true;
-}
 __device__ __forceinline__ bool fx_weak(const FxShared& sm, const int (&sE)[8][kSitesPerBlock], int site, int spin,
                                         int c) {
     int hops = 0, top = 0;
@@ -315,10 +295,30 @@ __device__ __forceinline__ bool fx_tile(const StencilArgs& a, int64_t base, int 
     }
     if (KEEP) {
         if (!__syncthreads_or(weak)) return false;
+        // A component is weak for nothing if its inputs are zero (what fixed point gives,
+        // zero, is then exact): every warp looks at the inputs of its hop.
+        int(&live)[4][kSitesPerBlock] = *(int(*)[4][kSitesPerBlock])sm.hop;
+        if (threadIdx.x < 4 * kSitesPerBlock) live[warp][lane] = 0;
+        __syncthreads();
+        if (sE[w >> 1][lane] > 0) {
+            const double2* p = l < a.a1 ? a.inA + (int64_t)(l - (int)a.a0) * kSiteC : a.inB + (int64_t)(l - (int)a.a1) * kSiteC;
+#pragma unroll
+            for (int k = 0; k < NS; ++k) {
+                const int up = NS == 1 ? (w & 1) : k, lo = w < 8 ? 3 - up : 2 + up;
+                bool any = false;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const double2 u = __ldg(p + 3 * up + c), v = __ldg(p + 3 * lo + c);
+                    any |= u.x != 0.0 || u.y != 0.0 || v.x != 0.0 || v.y != 0.0;
+                }
+                if (any) live[up][lane] = live[lo][lane] = 1;
+            }
+        }
+        __syncthreads();
         bool keep = false;
 #pragma unroll 1
         for (int v = warp; v < 12; v += kFxThreads<NS> / 32)
-            if (weak >> v & 1u) keep |= !fx_silent(a, a.o0 + base + ((v % 3) * 32 + lane) / 3, v / 3);
+            if (weak >> v & 1u) keep |= live[v / 3][((v % 3) * 32 + lane) / 3] != 0;
         return __syncthreads_or(keep);
     }
     __syncthreads();
