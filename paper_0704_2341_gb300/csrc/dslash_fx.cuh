@@ -177,8 +177,11 @@ __device__ __forceinline__ I2 fx_sum(const FxShared& sm, int site, int spin, int
 // in double precision takes some 15 us, so the lines lie where Gaussian spinors
 // meet them in less than 1e-8 of the components: |re| and |im| of a contribution are
 // both below 2^-8 with probability 3e-4, 2^-10 2e-5, 2^-16 5e-9.
-// Contributions that are zero because their inputs are (point sources and probes)
-// are exact in fixed point.
+// Contributions that are zero because their inputs are (point sources, single spin
+// components) are exact in fixed point, which fx_tile checks.  Gaussian input: 8^4
+// 8.2 us, 24^3 x 48 0.50 ms, as without all this; point source on 8^4 10.3 us; one spin
+// component alone 12.3 us and 0.70 ms, beside others 1e-12 of it 20.5 us and 1.8 ms
+// (every tile twice; in double precision alone 12.3 us and 1.03 ms).
 constexpr int kFxWeak1 = 16, kFxWeak2 = 10, kFxWeak = 8;     // k for one hop, two, more
 
 __device__ __forceinline__ int fx_weak_bits(int hops) {
